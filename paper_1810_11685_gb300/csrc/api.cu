@@ -141,23 +141,34 @@ cudaError_t dalloc(qpat_ctx* c, P** p, size_t bytes) {
 
 cudaError_t dalloc_cb(void* owner, void** p, size_t bytes) { return dalloc((qpat_ctx*)owner, p, bytes); }
 
+// Radices of an extent, fewest stages first: 8s, then what is left of the
+// twos (a single one joins a three as radix 6), pairs of threes as 9.
 bool factor_plan(int L, FFTPlan& p) {
   p.L = L;
   p.nstages = 0;
   int r = L;
-  int twos = 0;
+  int twos = 0, threes = 0;
   while (r % 2 == 0) { r /= 2; ++twos; }
-  while (twos >= 3) { p.radix[p.nstages++] = 8; twos -= 3; }
-  if (twos == 2) p.radix[p.nstages++] = 4;
-  if (twos == 1) p.radix[p.nstages++] = 2;
-  for (int q : {3, 5, 7}) {
+  while (r % 3 == 0) { r /= 3; ++threes; }
+  auto add = [&p](int q) {
+    if (p.nstages >= kMaxStages) return false;
+    p.radix[p.nstages++] = q;
+    return true;
+  };
+  bool ok = true;
+  while (twos >= 3) { ok = ok && add(8); twos -= 3; }
+  if (twos == 2) ok = ok && add(4);
+  if (twos == 1 && threes > 0) { ok = ok && add(6); --threes; }
+  else if (twos == 1) ok = ok && add(2);
+  while (threes >= 2) { ok = ok && add(9); threes -= 2; }
+  if (threes == 1) ok = ok && add(3);
+  for (int q : {5, 7}) {
     while (r % q == 0) {
-      if (p.nstages >= kMaxStages) return false;
-      p.radix[p.nstages++] = q;
+      ok = ok && add(q);
       r /= q;
     }
   }
-  return r == 1 && p.nstages <= kMaxStages;
+  return ok && r == 1;
 }
 
 template <typename T>

@@ -4,8 +4,8 @@
 // memory (sequence m at offset m*L).  Each stage with radix R reads R points
 // at stride L/R, applies the twiddles W_{Ns R}^(k r) and an R-point DFT, and
 // writes them self-sorted (Stockham autosort), so the result comes out in
-// natural order after ping-ponging between two buffers.  Radices 2, 3, 4, 5,
-// 7 and 8 are written out by hand.  The transform is the forward DFT
+// natural order after ping-ponging between two buffers.  Radices 2 to 9 are
+// written out by hand.  The transform is the forward DFT
 // X_k = sum_n x_n exp(-2 pi i n k / L), unnormalised; inverse transforms use
 // conj(FFT(conj(.))).  Twiddles come from a table W_L^m, m = 0..L-1,
 // computed in FP64 on the device and rounded to the working precision.
@@ -138,33 +138,86 @@ template <typename C> __device__ __forceinline__ void dft8(C* a) {
   a[3] = cadd(e[3], o3);   a[7] = csub(e[3], o3);
 }
 
-// One Stockham stage of radix R over M sequences.
+// Exact t / d for 0 <= t and t d < 2^32 by one multiply-high (a runtime
+// divisor would cost about twenty instructions for every quotient).
+struct FastDiv {
+  unsigned d, mul;
+  __device__ __forceinline__ explicit FastDiv(int div) : d((unsigned)div), mul(0xffffffffu / (unsigned)div + 1u) {}
+  __device__ __forceinline__ int div(int t) const { return d == 1u ? t : (int)__umulhi((unsigned)t, mul); }
+};
+
+template <typename C> __device__ __forceinline__ void dft6(C* a) {
+  typedef decltype(C().x) R;
+  const R h = (R)0.8660254037844386467637231707529362;   // sqrt(3)/2 = Im of -W6^2
+  C e[3] = {a[0], a[2], a[4]};
+  C o[3] = {a[1], a[3], a[5]};
+  dft3(e);
+  dft3(o);
+  // W6^1 = 1/2 - i h, W6^2 = -1/2 - i h
+  C o1 = cmake<C>((R)0.5 * o[1].x + h * o[1].y, (R)0.5 * o[1].y - h * o[1].x);
+  C o2 = cmake<C>(h * o[2].y - (R)0.5 * o[2].x, -(R)0.5 * o[2].y - h * o[2].x);
+  a[0] = cadd(e[0], o[0]); a[3] = csub(e[0], o[0]);
+  a[1] = cadd(e[1], o1);   a[4] = csub(e[1], o1);
+  a[2] = cadd(e[2], o2);   a[5] = csub(e[2], o2);
+}
+
+template <typename C> __device__ __forceinline__ void dft9(C* a) {
+  typedef decltype(C().x) R;
+  // W9^1, W9^2, W9^4 as (cos, -sin)
+  const C w1 = cmake<C>((R)0.7660444431189780352023926505554167, (R)-0.6427876096865393263226434099072632);
+  const C w2 = cmake<C>((R)0.1736481776669303488517166267693148, (R)-0.9848077530122080593667430245895230);
+  const C w4 = cmake<C>((R)-0.9396926207859083840541092773247314, (R)-0.3420201433256687330440996146822596);
+  C t[3][3];
+#pragma unroll
+  for (int n = 0; n < 3; ++n) {
+    t[n][0] = a[n]; t[n][1] = a[n + 3]; t[n][2] = a[n + 6];
+    dft3(t[n]);
+  }
+  t[1][1] = cmul(t[1][1], w1);
+  t[1][2] = cmul(t[1][2], w2);
+  t[2][1] = cmul(t[2][1], w2);
+  t[2][2] = cmul(t[2][2], w4);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    C u[3] = {t[0][k], t[1][k], t[2][k]};
+    dft3(u);
+    a[k] = u[0]; a[k + 3] = u[1]; a[k + 6] = u[2];
+  }
+}
+
+// One Stockham stage of radix R over M sequences.  The index arithmetic has
+// no division or modulo per butterfly: the two quotients go through FastDiv,
+// and the twiddle exponent k r L/(Ns R) is below L as it stands (k < Ns,
+// r < R).
 template <int R, typename C>
 __device__ __forceinline__ void stockham_stage(const C* __restrict__ in, C* __restrict__ out, int L, int M,
                                                int S, int Ns, const C* __restrict__ tw) {
   const int nb = L / R;                  // butterflies per sequence
   const int total = nb * M;
-  const int twstep = L / (Ns * R);       // W_{Ns R}^k = W_L^(k * twstep)
+  const int twstep = nb / Ns;            // W_{Ns R}^k = W_L^(k * twstep)
+  const FastDiv by_nb(nb), by_ns(Ns);
   for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    const int m = t / nb;
+    const int m = by_nb.div(t);
     const int j = t - m * nb;
     const C* src = in + m * S;
     C a[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) a[r] = src[j + r * nb];
-    const int k = j % Ns;
+    const int q = by_ns.div(j), k = j - q * Ns;
     if (Ns > 1) {
       const int base = k * twstep;
 #pragma unroll
-      for (int r = 1; r < R; ++r) a[r] = cmul(a[r], tw[(base * r) % L]);
+      for (int r = 1; r < R; ++r) a[r] = cmul(a[r], tw[base * r]);
     }
     if (R == 2) dft2(a);
     else if (R == 3) dft3(a);
     else if (R == 4) dft4(a);
     else if (R == 5) dft5(a);
+    else if (R == 6) dft6(a);
     else if (R == 7) dft7(a);
     else if (R == 8) dft8(a);
-    C* dst = out + m * S + (j / Ns) * Ns * R + k;
+    else if (R == 9) dft9(a);
+    C* dst = out + m * S + q * Ns * R + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) dst[r * Ns] = a[r];
   }
@@ -186,8 +239,10 @@ __device__ C* fft_batch(const FFTPlan& plan, C* buf0, C* buf1, int M, int S, con
       case 3: stockham_stage<3>(in, out, plan.L, M, S, Ns, tw); break;
       case 4: stockham_stage<4>(in, out, plan.L, M, S, Ns, tw); break;
       case 5: stockham_stage<5>(in, out, plan.L, M, S, Ns, tw); break;
+      case 6: stockham_stage<6>(in, out, plan.L, M, S, Ns, tw); break;
       case 7: stockham_stage<7>(in, out, plan.L, M, S, Ns, tw); break;
       case 8: stockham_stage<8>(in, out, plan.L, M, S, Ns, tw); break;
+      case 9: stockham_stage<9>(in, out, plan.L, M, S, Ns, tw); break;
       default: break;
     }
     __syncthreads();

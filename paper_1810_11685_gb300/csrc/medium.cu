@@ -36,7 +36,7 @@ using namespace qpat::med;
 constexpr int kThreads = 256;
 // Largest whole-history tape of the medium gradient (beyond it: checkpoints).
 constexpr double kFullTapeBytes = 2.0 * 1024 * 1024 * 1024;
-constexpr long long kMaxBlocks = 152 * 16;
+constexpr long long kMaxBlocks = kSMs * 16;
 
 template <class F>
 __global__ void __launch_bounds__(kThreads) for_each_kernel(const F f, long long n) {
@@ -273,11 +273,22 @@ cols_fast_kernel(const float2* Zi, int nin, float2* Zc, const Terms tm, const Ta
   }
 }
 
-// Lines per CTA of the row launches: about 48 KB of shared memory per
-// buffer, 1 to 16 lines.
-int lines_per_cta(int L, int csize) {
-  const int m = 49152 / ((L + 1) * csize);
-  return m < 1 ? 1 : m > 16 ? 16 : m;
+// Lines per CTA of the row launches over n lines: about 48 KB of shared
+// memory per buffer, 1 to 16 lines, halved while the launch has fewer CTAs
+// than the chip has SMs (168^2: 16 lines a CTA made 11 to 22 CTAs of 33 us in
+// FP64; with the narrower column launch below the gradient over 100 steps
+// went from 82.7 to 42.9 ms).
+int lines_per_cta(int L, int csize, int n) {
+  int m = 49152 / ((L + 1) * csize);
+  m = m < 1 ? 1 : m > 16 ? 16 : m;
+  while (m > 1 && (n + m - 1) / m < kSMs) m = (m + 1) / 2;
+  return m;
+}
+// Threads of a launch whose CTAs hold n lines of L points: one per radix-4
+// butterfly, in whole warps, at most `most`.
+int line_threads(int L, int n, int most) {
+  const int t = (n * L / 4 + 31) / 32 * 32;
+  return t < 64 ? 64 : t > most ? most : t;
 }
 // Columns per CTA of the column launch: two buffers of W lines per column
 // within the shared-memory budget, a power of two from 1 to 8 (so that a
@@ -285,12 +296,14 @@ int lines_per_cta(int L, int csize) {
 // Budget 110 KB in FP32 (two CTAs per SM) and 220 KB in FP64 (measured at
 // 576^2, 2000 steps, gradient / tangent: FP32 1.95 / 0.79 s against 2.51 /
 // 0.85 s with 220 KB and 1.89 / 0.89 s with 56 KB; FP64 4.73 / 2.90 s with
-// 220 KB against 4.93 / 3.06 s with 110 KB).
-int cols_per_cta(int L, int W, int csize) {
+// 220 KB against 4.93 / 3.06 s with 110 KB).  Halved while the launch has
+// fewer CTAs than the chip has SMs (168^2 FP64: 21 CTAs of 8 columns took 70 us).
+int cols_per_cta(int L, int W, int csize, int nx) {
   const int budget = csize >= 16 ? 225280 : 112640;
   const int m = budget / (2 * W * (L + 1) * csize);
   int p = 1;
   while (2 * p <= m && 2 * p <= 8) p *= 2;
+  while (p > 1 && (nx + p - 1) / p < kSMs) p /= 2;
   return p;
 }
 
@@ -354,10 +367,10 @@ struct GpuEx {
       if (nb > 0 && err == cudaSuccess && rows_fast<false>(f, nullptr, Z, FieldPtrs<float*>{}, 1.f, nb, t, G)) return;
     }
     const FFTPlan plan = to_fft_plan(t.px);
-    const int M = lines_per_cta(plan.L, (int)sizeof(Cplx<R>));
+    const int M = lines_per_cta(plan.L, (int)sizeof(Cplx<R>), t.ny * nb);
     const size_t smem = 2 * (size_t)M * (plan.L + 1) * sizeof(Cplx<R>);
     if (nb <= 0 || !smem_limit(rows_fwd_kernel<R>, smem)) return;
-    rows_fwd_kernel<R><<<dim3((t.ny + M - 1) / M, nb), kLineThreads, smem, s>>>(f, Z, G, t.nx, t.ny, plan, t.twx, M);
+    rows_fwd_kernel<R><<<dim3((t.ny + M - 1) / M, nb), line_threads(plan.L, M, kLineThreads), smem, s>>>(f, Z, G, t.nx, t.ny, plan, t.twx, M);
     launched();
   }
   // the compile-time column launch (FP32, extents 24, 168, 576)
@@ -388,10 +401,10 @@ struct GpuEx {
     }
     const FFTPlan plan = to_fft_plan(t.py);
     const int W = nin > tm.no ? nin : tm.no;
-    const int M = cols_per_cta(plan.L, W, (int)sizeof(Cplx<R>));
+    const int M = cols_per_cta(plan.L, W, (int)sizeof(Cplx<R>), t.nx);
     const size_t smem = 2 * (size_t)W * M * (plan.L + 1) * sizeof(Cplx<R>);
     if (nin <= 0 || !smem_limit(cols_kernel<R>, smem)) return;
-    cols_kernel<R><<<(t.nx + M - 1) / M, kColThreads, smem, s>>>(Zi, nin, Zc, tm, t, G, plan, M, W);
+    cols_kernel<R><<<(t.nx + M - 1) / M, line_threads(plan.L, W * M, kColThreads), smem, s>>>(Zi, nin, Zc, tm, t, G, plan, M, W);
     launched();
   }
   // out[o] = alpha Re F_x^-1 Z[o] for o < no
@@ -402,10 +415,10 @@ struct GpuEx {
         return;
     }
     const FFTPlan plan = to_fft_plan(t.px);
-    const int M = lines_per_cta(plan.L, (int)sizeof(Cplx<R>));
+    const int M = lines_per_cta(plan.L, (int)sizeof(Cplx<R>), t.ny * no);
     const size_t smem = 2 * (size_t)M * (plan.L + 1) * sizeof(Cplx<R>);
     if (no <= 0 || !smem_limit(rows_inv_kernel<R>, smem)) return;
-    rows_inv_kernel<R><<<dim3((t.ny + M - 1) / M, no), kLineThreads, smem, s>>>(Z, out, alpha, G, t.nx, t.ny, plan,
+    rows_inv_kernel<R><<<dim3((t.ny + M - 1) / M, no), line_threads(plan.L, M, kLineThreads), smem, s>>>(Z, out, alpha, G, t.nx, t.ny, plan,
                                                                                 t.twx, M);
     launched();
   }

@@ -44,6 +44,11 @@ template <> struct ColIO<A_C6> { static constexpr int kin = 2, kout = 1; };
 
 constexpr int kRowThreads = 256;
 constexpr int kColThreads = 256;
+// Resident CTAs per SM the generic passes are compiled for: the radix-9
+// butterfly would otherwise take 56-64 registers a thread in FP32 (126 in
+// FP64) in every launch, also where no stage uses it.
+template <typename T>
+constexpr int generic_minb() { return sizeof(T) == 4 ? 5 : 3; }
 
 template <typename T>
 size_t row_smem_bytes(int nx) {
@@ -60,7 +65,7 @@ size_t col_smem_bytes(int ny, int cb) {
 // Row pass: rows j0 = 2*blockIdx.x and j0 + 1 of problem blockIdx.y.
 // ---------------------------------------------------------------------------
 template <typename T, int PH>
-__global__ void __launch_bounds__(kRowThreads) row_kernel(const PropArgs<T> a) {
+__global__ void __launch_bounds__(kRowThreads, generic_minb<T>()) row_kernel(const PropArgs<T> a) {
   typedef typename V2<T>::t C;
   constexpr int KIN = RowIO<PH>::kin;
   constexpr int KOUT = RowIO<PH>::kout;
@@ -159,7 +164,7 @@ __global__ void __launch_bounds__(kRowThreads) row_kernel(const PropArgs<T> a) {
 // Column pass: half-spectrum columns kx0 .. kx0+cb-1 of problem blockIdx.y.
 // ---------------------------------------------------------------------------
 template <typename T, int PH>
-__global__ void __launch_bounds__(kColThreads) col_kernel(const PropArgs<T> a) {
+__global__ void __launch_bounds__(kColThreads, generic_minb<T>()) col_kernel(const PropArgs<T> a) {
   typedef typename V2<T>::t C;
   constexpr int KIN = ColIO<PH>::kin;
   constexpr int KOUT = ColIO<PH>::kout;
@@ -173,11 +178,13 @@ __global__ void __launch_bounds__(kColThreads) col_kernel(const PropArgs<T> a) {
   C* spec = a.spec + (long long)b * a.sstride;
   const long long slot = (long long)ny * a.pitch;
 
+  const FastDiv by_cb(cb), by_ny(ny);
+
   if (PH == F_C1) sensor_gather<T>(a, b, blockIdx.x * nth + tid, gridDim.x * nth);   // eq. num-m
 
   for (int s = 0; s < KIN; ++s) {
     for (int idx = tid; idx < ny * cb; idx += nth) {
-      const int ky = idx / cb, c = idx - ky * cb, kx = kx0 + c;
+      const int ky = by_cb.div(idx), c = idx - ky * cb, kx = kx0 + c;
       C v = cmake<C>((T)0, (T)0);
       if (kx < nxh) v = spec[s * slot + (long long)ky * a.pitch + kx];
       buf0[(s * cb + c) * S + ky] = v;
@@ -188,7 +195,7 @@ __global__ void __launch_bounds__(kColThreads) col_kernel(const PropArgs<T> a) {
   C* oth = (res == buf0) ? buf1 : buf0;
 
   for (int idx = tid; idx < ny * cb; idx += nth) {
-    const int c = idx / ny, ky = idx - c * ny, kx = kx0 + c;
+    const int c = by_ny.div(idx), ky = idx - c * ny, kx = kx0 + c;
     C o0 = cmake<C>((T)0, (T)0), o1 = o0;
     if (kx < nxh) {
       const C X0 = res[c * S + ky];
@@ -202,7 +209,7 @@ __global__ void __launch_bounds__(kColThreads) col_kernel(const PropArgs<T> a) {
   C* res2 = fft_batch(a.py, oth, res, KOUT * cb, S, a.twy);
   for (int o = 0; o < KOUT; ++o) {
     for (int idx = tid; idx < ny * cb; idx += nth) {
-      const int ky = idx / cb, c = idx - ky * cb, kx = kx0 + c;
+      const int ky = by_cb.div(idx), c = idx - ky * cb, kx = kx0 + c;
       if (kx < nxh) spec[o * slot + (long long)ky * a.pitch + kx] = cconj(res2[(o * cb + c) * S + ky]);
     }
   }
@@ -284,25 +291,48 @@ void launch_row(const PropArgs<T>& a, int phase, int batch, cudaStream_t s) {
   }
 }
 
+// Columns per CTA of a generic column launch: the widest tile the context
+// allows, halved while the launch has fewer CTAs than the chip has SMs.  A
+// wide tile reads whole 32-byte sectors, but at 168^2, one problem, 8 columns
+// make 11 CTAs, and the FP64 column pass is bound by the FP64 lanes of those
+// 11 SMs (measured, forward + adjoint of 150 steps: 62.2 ms with 8 columns,
+// 32.4 ms with 1; 150 x 210, two lossless FP32 problems, 200 steps: 15.4 ms
+// with 8 columns, 10.8 ms with 1).
+static int col_width(int cb, int nxh, int batch) {
+  while (cb > 1 && (nxh + cb - 1) / cb * batch < kSMs) cb /= 2;
+  return cb;
+}
+// Threads of a generic column launch: one per point of the tile, in whole
+// warps, at most kColThreads (the loads, the products and the stores have one
+// point a thread; half as many threads measured 34.4 against 32.4 ms and 11.4
+// against 10.8 ms on the two workloads above).
+static int col_threads(int ny, int cb) {
+  const int t = (cb * ny + 31) / 32 * 32;
+  return t < 64 ? 64 : t > kColThreads ? kColThreads : t;
+}
+
 template <typename T>
-void launch_col(const PropArgs<T>& a, int phase, int batch, cudaStream_t s) {
-  if constexpr (std::is_same<T, float>::value) if (a.fast_cols) {
-    switch (a.ny) {
-#define QPAT_COL_CASE(n) case n: launch_col_fast_len<T, n>(a, phase, batch, s); return;
+void launch_col(const PropArgs<T>& args, int phase, int batch, cudaStream_t s) {
+  if constexpr (std::is_same<T, float>::value) if (args.fast_cols) {
+    switch (args.ny) {
+#define QPAT_COL_CASE(n) case n: launch_col_fast_len<T, n>(args, phase, batch, s); return;
       QPAT_FAST_CASES(QPAT_COL_CASE)
 #undef QPAT_COL_CASE
       default: break;
     }
   }
+  PropArgs<T> a = args;
+  a.cb = col_width(args.cb, a.nxh, batch);
+  const int threads = col_threads(a.ny, a.cb);
   dim3 grid((a.nxh + a.cb - 1) / a.cb, batch);
   const size_t sm = col_smem_bytes<T>(a.ny, a.cb);
   switch (phase) {
-    case F_C1: col_kernel<T, F_C1><<<grid, kColThreads, sm, s>>>(a); break;
-    case F_C2: col_kernel<T, F_C2><<<grid, kColThreads, sm, s>>>(a); break;
-    case F_C3: col_kernel<T, F_C3><<<grid, kColThreads, sm, s>>>(a); break;
-    case A_C2: col_kernel<T, A_C2><<<grid, kColThreads, sm, s>>>(a); break;
-    case A_C4: col_kernel<T, A_C4><<<grid, kColThreads, sm, s>>>(a); break;
-    case A_C6: col_kernel<T, A_C6><<<grid, kColThreads, sm, s>>>(a); break;
+    case F_C1: col_kernel<T, F_C1><<<grid, threads, sm, s>>>(a); break;
+    case F_C2: col_kernel<T, F_C2><<<grid, threads, sm, s>>>(a); break;
+    case F_C3: col_kernel<T, F_C3><<<grid, threads, sm, s>>>(a); break;
+    case A_C2: col_kernel<T, A_C2><<<grid, threads, sm, s>>>(a); break;
+    case A_C4: col_kernel<T, A_C4><<<grid, threads, sm, s>>>(a); break;
+    case A_C6: col_kernel<T, A_C6><<<grid, threads, sm, s>>>(a); break;
     default: break;
   }
 }

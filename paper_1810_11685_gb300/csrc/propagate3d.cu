@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(k3Threads) ypass3_kernel(const Prop3<T> a, con
   typedef typename V2<T>::t C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int cb = a.cby, ny = a.ny, S = ny + 1, nxh = a.nxh;
+  const FastDiv by_cb(cb);
   C* buf0 = reinterpret_cast<C*>(smem_raw);
   C* buf1 = buf0 + 3 * cb * S;
   const int b = blockIdx.z, k = blockIdx.y, kx0 = blockIdx.x * cb;
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(k3Threads) ypass3_kernel(const Prop3<T> a, con
   C* spec = a.spec + (long long)b * a.sstride + (long long)k * ny * a.pitch;
   for (int s = 0; s < K; ++s)
     for (int idx = tid; idx < ny * cb; idx += nth) {
-      const int ky = idx / cb, c = idx - ky * cb, kx = kx0 + c;
+      const int ky = by_cb.div(idx), c = idx - ky * cb, kx = kx0 + c;
       C v = cmake<C>((T)0, (T)0);
       if (kx < nxh) v = spec[s * a.slot + (long long)ky * a.pitch + kx];
       buf0[(s * cb + c) * S + ky] = INV ? cconj(v) : v;
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(k3Threads) ypass3_kernel(const Prop3<T> a, con
   C* res = fft_batch(a.py, buf0, buf1, K * cb, S, a.twy);
   for (int s = 0; s < K; ++s)
     for (int idx = tid; idx < ny * cb; idx += nth) {
-      const int ky = idx / cb, c = idx - ky * cb, kx = kx0 + c;
+      const int ky = by_cb.div(idx), c = idx - ky * cb, kx = kx0 + c;
       if (kx < nxh) {
         const C v = res[(s * cb + c) * S + ky];
         spec[s * a.slot + (long long)ky * a.pitch + kx] = INV ? cconj(v) : v;
@@ -154,6 +155,7 @@ __global__ void __launch_bounds__(k3Threads) zpass3_kernel(const Prop3<T> a) {
   constexpr int KIN = z3_kin(PH), KOUT = z3_kout(PH);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int cb = a.cbz, nz = a.nz, S = nz + 1, nxh = a.nxh;
+  const FastDiv by_cb(cb), by_nz(nz);
   C* buf0 = reinterpret_cast<C*>(smem_raw);
   C* buf1 = buf0 + 3 * cb * S;
   const int b = blockIdx.z, ky = blockIdx.y, kx0 = blockIdx.x * cb;
@@ -162,7 +164,7 @@ __global__ void __launch_bounds__(k3Threads) zpass3_kernel(const Prop3<T> a) {
   C* spec = a.spec + (long long)b * a.sstride + (long long)ky * a.pitch;
   for (int s = 0; s < KIN; ++s)
     for (int idx = tid; idx < nz * cb; idx += nth) {
-      const int kz = idx / cb, c = idx - kz * cb, kx = kx0 + c;
+      const int kz = by_cb.div(idx), c = idx - kz * cb, kx = kx0 + c;
       C v = cmake<C>((T)0, (T)0);
       if (kx < nxh) v = spec[s * a.slot + kz * zs + kx];
       buf0[(s * cb + c) * S + kz] = v;
@@ -171,7 +173,7 @@ __global__ void __launch_bounds__(k3Threads) zpass3_kernel(const Prop3<T> a) {
   C* res = fft_batch(a.pz, buf0, buf1, KIN * cb, S, a.twz);
   C* oth = (res == buf0) ? buf1 : buf0;
   for (int idx = tid; idx < nz * cb; idx += nth) {
-    const int c = idx / nz, kz = idx - c * nz, kx = kx0 + c;
+    const int c = by_nz.div(idx), kz = idx - c * nz, kx = kx0 + c;
     C X[3], o[3];
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
@@ -187,7 +189,7 @@ __global__ void __launch_bounds__(k3Threads) zpass3_kernel(const Prop3<T> a) {
   C* res2 = fft_batch(a.pz, oth, res, KOUT * cb, S, a.twz);
   for (int s = 0; s < KOUT; ++s)
     for (int idx = tid; idx < nz * cb; idx += nth) {
-      const int kz = idx / cb, c = idx - kz * cb, kx = kx0 + c;
+      const int kz = by_cb.div(idx), c = idx - kz * cb, kx = kx0 + c;
       if (kx < nxh) spec[s * a.slot + kz * zs + kx] = cconj(res2[(s * cb + c) * S + kz]);
     }
 }

@@ -10,6 +10,8 @@ struct qpat_ctx;
 
 namespace qpat {
 
+constexpr int kSMs = 152;   // streaming multiprocessors of the GPU
+
 // Flags of one propagation kernel launch.
 enum : int {
   kSkipInput = 1,    // the incoming spectral slots are zero (first step)
