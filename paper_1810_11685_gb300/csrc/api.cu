@@ -819,6 +819,8 @@ qpat_status qpat_create(const qpat_config* cfg, const qpat_medium* med, const do
   QCKC(dalloc(c, &w.mu, B * N * sizeof(double)));
   QCKC(dalloc(c, &w.partial, (size_t)B * kPCGBlocks * 4 * sizeof(double)));
   QCKC(dalloc(c, &w.scal, (size_t)B * 8 * sizeof(double)));
+  QCKC(dalloc(c, &w.count, (size_t)B * sizeof(unsigned)));
+  QCKC(cudaMemset(w.count, 0, (size_t)B * sizeof(unsigned)));
   w.use_graphs = !c->cfg.no_graphs;
   if (!c->cfg.da_jacobi) {
     c->mg.reset(new MGHierarchy());

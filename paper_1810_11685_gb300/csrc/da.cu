@@ -70,16 +70,21 @@ cudaError_t da_setup(DAArgs& a, double* d_diag0, double* d_cxf, double* d_cyf, d
 
 __global__ void rhs_sides_kernel(DAArgs a, unsigned mask, double* rhs) {
   const int b = blockIdx.y;
+  const int sz = a.n0 * a.n1;
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.N; g += gridDim.x * blockDim.x) {
+    const int k = g / sz, rem = g - k * sz, j = rem / a.n0, i = rem - j * a.n0;
+    const bool on[6] = {i == 0, i == a.n0 - 1, j == 0, j == a.n1 - 1, k == 0, k == a.n2 - 1};
     double v = 0.0;
-    for (int s = 0; s < 2 * a.dim; ++s)
-      if ((mask >> s) & 1u) v += a.bside[(long long)s * a.N + g];
+#pragma unroll
+    for (int s = 0; s < 6; ++s)                       // a side's coefficient is zero away from that side
+      if (s < 2 * a.dim && on[s] && ((mask >> s) & 1u)) v += a.bside[(long long)s * a.N + g];
     rhs[(long long)b * a.N + g] = v;
   }
 }
 
 cudaError_t da_rhs_from_sides(const DAArgs& a, unsigned mask, int batch, double* rhs, cudaStream_t s) {
-  rhs_sides_kernel<<<dim3(64, batch), kThreads, 0, s>>>(a, mask, rhs);
+  rhs_sides_kernel<<<dim3((unsigned)std::min(kPCGBlocks, (a.N + kThreads - 1) / kThreads), batch), kThreads, 0, s>>>(a, mask,
+                                                                                                                rhs);
   return cudaGetLastError();
 }
 
@@ -284,6 +289,9 @@ cudaError_t mg_setup(MGHierarchy& h, const DAArgs& fine, const double* d_kappa, 
     if ((e = alloc(owner, (void**)&L.x2, bytes)) != cudaSuccess) return e;
     if (l > 0 && (e = alloc(owner, (void**)&L.x, bytes)) != cudaSuccess) return e;
     if (l > 0 && (e = alloc(owner, (void**)&L.b, bytes)) != cudaSuccess) return e;
+    // (level 0 uses the PCG work vectors for these)
+    if (l > 0 && (e = alloc(owner, (void**)&L.d, bytes)) != cudaSuccess) return e;
+    if (l > 0 && (e = alloc(owner, (void**)&L.w, bytes)) != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }
@@ -302,169 +310,605 @@ cudaError_t mg_rekappa(MGHierarchy& h, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// x_out = x_in + omega D^-1 (b - A x_in); x_in = 0 when first
-__global__ void mg_jacobi_kernel(DAArgs a, const double* mu, const double* xin, const double* b, double* xout,
-                                 double omega, int first) {
-  const long long o = (long long)blockIdx.y * a.N;
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.N; g += gridDim.x * blockDim.x) {
-    const double d = a.diag0[g] + mu[o + g] * a.hd;
-    if (first) {
-      xout[o + g] = omega * b[o + g] / d;
-    } else {
-      const double ax = apply_A(a, mu + o, xin + o, g, a.hd);
-      xout[o + g] = xin[o + g] + omega * (b[o + g] - ax) / d;
-    }
+// ---- V-cycle and multigrid-preconditioned iteration ----------------------------
+// GB300 has two FP64 fused multiply-adds per clock and SM, so on large grids
+// these kernels are bound by FP64 arithmetic as much as by memory, and on
+// small ones by the number of launches.  Hence: the smoother multiplies by a
+// stored omega / d instead of dividing (a division is about ten FP64
+// instructions; a sweep is 2 dim + 2); the first sweep from zero is part of
+// the kernel that makes the right-hand side, the prolongation part of the
+// coarse level's last sweep, and every inner product is finished by the last
+// block of the kernel that forms it; a thread takes two adjacent cells with
+// 16-byte loads; all levels of at most kSmallCells cells run in one CTA per
+// problem, in shared memory; and a converged problem's blocks return at once.
+// Measured on GB300: 512^2, 8 problems 12.2 -> 4.9 ms; 128^2, one problem 2.6 -> 1.3 ms; 90^2
+// (stops at 45^2) 14.7 -> 3.2 ms; the forward map on 256^3 with 24 time steps 130 -> 81 ms.
+
+// One level of one solve, as the kernels see it.
+struct LevDev {
+  int n0, n1, n2, N;
+  const double *cx, *cy, *cz, *d, *w;
+  double *x, *x2, *b;
+};
+
+static LevDev mg_dev(const MGLevel& L, const PCGWork&) {
+  return LevDev{L.A.n0, L.A.n1, L.A.n2, L.A.N, L.A.cxf, L.A.cyf, L.A.czf, L.d, L.w, L.x, L.x2, L.b};
+}
+
+// Launch shape of a level: TX x TY threads, a thread taking VEC adjacent cells
+// of a grid line (VEC = 2 where lines are even), blocks striding over lines.
+// It depends on the level only, so a problem's sums are the same in any batch.
+struct MGGrid {
+  dim3 grid, block;
+  int vec;
+};
+static MGGrid mg_grid(const DAArgs& a, int batch) {
+  MGGrid g;
+  g.vec = a.n0 % 2 == 0 ? 2 : 1;
+  int tx = 8;
+  while (tx < 64 && tx < a.n0 / g.vec) tx *= 2;
+  const int ty = kThreads / tx, lines = a.n1 * a.n2;
+  g.block = dim3(tx, ty);
+  g.grid = dim3((unsigned)std::min(kPCGBlocks, (lines + ty - 1) / ty), batch);
+  return g;
+}
+static dim3 mg_blocks(int N, int batch) {
+  return dim3((unsigned)std::min(kPCGBlocks, (N + kThreads - 1) / kThreads), batch);
+}
+#define MG_DISPATCH(A_, kernel, g_, s_, ...)                                                \
+  do {                                                                                      \
+    if ((A_).dim == 3) {                                                                    \
+      if ((g_).vec == 2) kernel<3, 2><<<(g_).grid, (g_).block, 0, s_>>>(__VA_ARGS__);       \
+      else kernel<3, 1><<<(g_).grid, (g_).block, 0, s_>>>(__VA_ARGS__);                     \
+    } else {                                                                                \
+      if ((g_).vec == 2) kernel<2, 2><<<(g_).grid, (g_).block, 0, s_>>>(__VA_ARGS__);       \
+      else kernel<2, 1><<<(g_).grid, (g_).block, 0, s_>>>(__VA_ARGS__);                     \
+    }                                                                                       \
+  } while (0)
+
+template <int VEC>
+struct Cells {
+  double v[VEC];
+};
+template <int VEC>
+__device__ __forceinline__ Cells<VEC> ld(const double* p) {
+  Cells<VEC> c;
+  if constexpr (VEC == 2) {
+    const double2 t = *reinterpret_cast<const double2*>(p);
+    c.v[0] = t.x;
+    c.v[1] = t.y;
+  } else {
+    c.v[0] = *p;
+  }
+  return c;
+}
+template <int VEC>
+__device__ __forceinline__ void st(double* p, const Cells<VEC>& c) {
+  if constexpr (VEC == 2) *reinterpret_cast<double2*>(p) = make_double2(c.v[0], c.v[1]);
+  else *p = c.v[0];
+}
+
+// body(g, i, j, k) for the VEC-cell groups of a level of blockIdx.y's problem.
+template <int DIM, int VEC, class F>
+__device__ __forceinline__ void for_groups(int n0, int n1, int n2, F&& body) {
+  const int lines = n1 * n2;
+  for (int line = blockIdx.x * blockDim.y + threadIdx.y; line < lines; line += gridDim.x * blockDim.y) {
+    const int k = DIM == 3 ? line / n1 : 0, j = DIM == 3 ? line - k * n1 : line;
+    for (int i = threadIdx.x * VEC; i < n0; i += blockDim.x * VEC) body(line * n0 + i, i, j, k);
   }
 }
 
-// b_c[I] = sum over the children i of I of (b_f - A_f x_f)[i]
-__global__ void mg_restrict_kernel(DAArgs f, const double* mu, const double* x, const double* bf, double* bc,
-                                   int cn0, int cn1, int cn2) {
-  const long long Nc = (long long)cn0 * cn1 * cn2;
-  const long long of = (long long)blockIdx.y * f.N, oc = (long long)blockIdx.y * Nc;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < Nc; t += (long long)gridDim.x * blockDim.x) {
-    const int I = (int)(t % cn0), J = (int)((t / cn0) % cn1), K = (int)(t / ((long long)cn0 * cn1));
+// c - A x at the VEC cells from g = (i, j, k); X receives x there.
+template <int DIM, int VEC>
+__device__ __forceinline__ Cells<VEC> residual(const LevDev& L, const double* d, const double* x, Cells<VEC> c, int g,
+                                               int i, int j, int k, Cells<VEC>& X) {
+  const int sy = L.n0, sz = L.n0 * L.n1;
+  X = ld<VEC>(x + g);
+  const Cells<VEC> D = ld<VEC>(d + g), cr = ld<VEC>(L.cx + g);
+  const double cl = i > 0 ? L.cx[g - 1] : 0.0, xl = i > 0 ? x[g - 1] : 0.0;
+  const double xr = i + VEC < L.n0 ? x[g + VEC] : 0.0;
+#pragma unroll
+  for (int v = 0; v < VEC; ++v) {
+    c.v[v] -= D.v[v] * X.v[v];
+    c.v[v] += (v ? cr.v[0] : cl) * (v ? X.v[0] : xl);
+    c.v[v] += cr.v[v] * (v + 1 < VEC ? X.v[VEC - 1] : xr);       // (zero coefficient at the last cell of a line)
+  }
+  if (j > 0) {
+    const Cells<VEC> f = ld<VEC>(L.cy + g - sy), y = ld<VEC>(x + g - sy);
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) c.v[v] += f.v[v] * y.v[v];
+  }
+  if (j < L.n1 - 1) {
+    const Cells<VEC> f = ld<VEC>(L.cy + g), y = ld<VEC>(x + g + sy);
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) c.v[v] += f.v[v] * y.v[v];
+  }
+  if (DIM == 3) {
+    if (k > 0) {
+      const Cells<VEC> f = ld<VEC>(L.cz + g - sz), y = ld<VEC>(x + g - sz);
+#pragma unroll
+      for (int v = 0; v < VEC; ++v) c.v[v] += f.v[v] * y.v[v];
+    }
+    if (k < L.n2 - 1) {
+      const Cells<VEC> f = ld<VEC>(L.cz + g), y = ld<VEC>(x + g + sz);
+#pragma unroll
+      for (int v = 0; v < VEC; ++v) c.v[v] += f.v[v] * y.v[v];
+    }
+  }
+  return c;
+}
+
+// Sum v over the launch's blocks of problem blockIdx.y, in a fixed order: true
+// (with the total in v) in thread 0 of the block that finishes last.
+__device__ __forceinline__ double block_sum(double v, double* sh) {
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if ((tid & 31) == 0) sh[tid >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (tid == 0)
+    for (int q = 0; q < kThreads / 32; ++q) t += sh[q];
+  return t;
+}
+__device__ __forceinline__ bool last_block_sum(double& v, const PCGWork& w) {
+  __shared__ double sh[kThreads / 32], sh2[kThreads / 32];
+  __shared__ bool last;
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x, b = blockIdx.y;
+  double* part = w.partial + (long long)b * kPCGBlocks * 4;
+  const double t = block_sum(v, sh);
+  if (tid == 0) {
+    part[blockIdx.x] = t;
+    __threadfence();
+    last = atomicAdd(&w.count[b], 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  double u = 0.0;
+  for (int q = tid; q < (int)gridDim.x; q += kThreads) u += __ldcg(part + q);
+  v = block_sum(u, sh2);
+  if (tid == 0) w.count[b] = 0;
+  return tid == 0;
+}
+__device__ __forceinline__ bool pcg_done(const PCGWork& w) { return w.scal[8 * blockIdx.y + 5] != 0.0; }
+
+// d = diag0 + mu h^dim and omega / d of a level.
+__global__ void mg_diag_kernel(DAArgs a, const double* mu, double omega, double* d, double* w) {
+  const long long o = (long long)blockIdx.y * a.N;
+  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.N; g += gridDim.x * blockDim.x) {
+    const double v = a.diag0[g] + mu[o + g] * a.hd;
+    d[o + g] = v;
+    w[o + g] = omega / v;
+  }
+}
+// The same on the next level, whose absorption is the mean of the children's.
+__global__ void mg_coarsen_kernel(DAArgs f, DAArgs c, const double* muf, double omega, double* muc, double* d,
+                                  double* w) {
+  const long long of = (long long)blockIdx.y * f.N, oc = (long long)blockIdx.y * c.N;
+  const double inv = f.dim == 3 ? 0.125 : 0.25;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < c.N; t += gridDim.x * blockDim.x) {
+    const int I = t % c.n0, J = (t / c.n0) % c.n1, K = t / (c.n0 * c.n1);
     double acc = 0.0;
     for (int dz = 0; dz < (f.dim == 3 ? 2 : 1); ++dz)
       for (int dy = 0; dy < 2; ++dy)
-        for (int dx = 0; dx < 2; ++dx) {
-          const int g = ((f.dim == 3 ? 2 * K + dz : 0) * f.n1 + 2 * J + dy) * f.n0 + 2 * I + dx;
-          acc += bf[of + g] - apply_A(f, mu + of, x + of, g, f.hd);
-        }
-    bc[oc + t] = acc;
+        for (int dx = 0; dx < 2; ++dx)
+          acc += muf[of + ((long long)(f.dim == 3 ? 2 * K + dz : 0) * f.n1 + 2 * J + dy) * f.n0 + 2 * I + dx];
+    const double m = acc * inv, v = c.diag0[t] + m * c.hd;
+    muc[oc + t] = m;
+    d[oc + t] = v;
+    w[oc + t] = omega / v;
   }
 }
 
-// x_f[i] += x_c[parent(i)]
-__global__ void mg_prolong_kernel(DAArgs f, const double* xc, double* xf, int cn0, int cn1, int cn2) {
-  const long long Nc = (long long)cn0 * cn1 * cn2;
-  const long long of = (long long)blockIdx.y * f.N, oc = (long long)blockIdx.y * Nc;
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < f.N; g += gridDim.x * blockDim.x) {
-    const int i = g % f.n0, j = (g / f.n0) % f.n1, k = g / (f.n0 * f.n1);
-    const long long pc = ((long long)(f.dim == 3 ? k / 2 : 0) * cn1 + j / 2) * cn0 + i / 2;
-    xf[of + g] += xc[oc + pc];
-  }
-}
-
-// All sweeps of the coarsest level in one CTA per problem (the level has at
-// most kCoarseCells cells): x = 0, then `sweeps` damped-Jacobi sweeps, the
-// result left in x.
-constexpr int kCoarseCells = 4096;
-__global__ void mg_coarse_kernel(DAArgs a, const double* mu, const double* b, double* x, double* x2, double omega,
-                                 int sweeps) {
-  const long long o = (long long)blockIdx.x * a.N;
-  double* cur = x + o;
-  double* nxt = x2 + o;
-  for (int g = threadIdx.x; g < a.N; g += blockDim.x)
-    cur[g] = omega * b[o + g] / (a.diag0[g] + mu[o + g] * a.hd);
-  for (int it = 1; it < sweeps; ++it) {
-    __syncthreads();
-    for (int g = threadIdx.x; g < a.N; g += blockDim.x) {
-      const double d = a.diag0[g] + mu[o + g] * a.hd;
-      nxt[g] = cur[g] + omega * (b[o + g] - apply_A(a, mu + o, cur, g, a.hd)) / d;
+// out = x + w (b - A x).  DOT: b . out into scal[slot] (level 0: r.z).
+// PROLONG: the result is not stored but added to its children in xf.
+enum SweepMode { kSweep, kSweepDot, kSweepProlong };
+template <int DIM, int VEC, int MODE>
+__device__ __forceinline__ void sweep_body(const LevDev& L, const double* xin, double* out, const PCGWork& w, int slot,
+                                           double* xf) {
+  if (pcg_done(w)) return;
+  const long long o = (long long)blockIdx.y * L.N;
+  const double *x = xin + o, *d = L.d + o;
+  double dot = 0.0;
+  for_groups<DIM, VEC>(L.n0, L.n1, L.n2, [&](int g, int i, int j, int k) {
+    const Cells<VEC> b = ld<VEC>(L.b + o + g), wd = ld<VEC>(L.w + o + g);
+    Cells<VEC> X, r = residual<DIM, VEC>(L, d, x, b, g, i, j, k, X);
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) {
+      r.v[v] = X.v[v] + wd.v[v] * r.v[v];
+      if (MODE == kSweepDot) dot += b.v[v] * r.v[v];
     }
+    if (MODE != kSweepProlong) {
+      st<VEC>(out + o + g, r);
+    } else {
+      const int f0 = 2 * L.n0, f1 = 2 * L.n1;
+      double* f = xf + (long long)blockIdx.y * L.N * (DIM == 3 ? 8 : 4);
+#pragma unroll
+      for (int v = 0; v < VEC; ++v)
+        for (int dz = 0; dz < (DIM == 3 ? 2 : 1); ++dz)
+          for (int dy = 0; dy < 2; ++dy) {
+            double2* q = reinterpret_cast<double2*>(f + ((long long)(DIM == 3 ? 2 * k + dz : 0) * f1 + 2 * j + dy) * f0 +
+                                                    2 * (i + v));
+            double2 t = *q;
+            t.x += r.v[v];
+            t.y += r.v[v];
+            *q = t;
+          }
+    }
+  });
+  if (MODE == kSweepDot) {
+    if (last_block_sum(dot, w)) w.scal[8 * blockIdx.y + slot] = dot;
+  }
+}
+template <int DIM, int VEC>
+__global__ void __launch_bounds__(kThreads) mg_sweep(LevDev L, const double* xin, double* out, PCGWork w) {
+  sweep_body<DIM, VEC, kSweep>(L, xin, out, w, 0, nullptr);
+}
+template <int DIM, int VEC>
+__global__ void __launch_bounds__(kThreads) mg_sweep_dot(LevDev L, const double* xin, double* out, PCGWork w, int slot) {
+  sweep_body<DIM, VEC, kSweepDot>(L, xin, out, w, slot, nullptr);
+}
+template <int DIM, int VEC>
+__global__ void __launch_bounds__(kThreads) mg_sweep_prolong(LevDev L, const double* xin, double* xf, PCGWork w) {
+  sweep_body<DIM, VEC, kSweepProlong>(L, xin, nullptr, w, 0, xf);
+}
+
+// b_c = sum over the children of (b - A x), and the first sweep from zero
+// there, x2_c = w_c b_c.  A thread takes one coarse cell (fine lines are even).
+template <int DIM>
+__global__ void __launch_bounds__(kThreads) mg_restrict(LevDev F, LevDev C, PCGWork w) {
+  if (pcg_done(w)) return;
+  const long long of = (long long)blockIdx.y * F.N, oc = (long long)blockIdx.y * C.N;
+  for_groups<DIM, 1>(C.n0, C.n1, C.n2, [&](int t, int I, int J, int K) {
+    double acc = 0.0;
+#pragma unroll
+    for (int dz = 0; dz < (DIM == 3 ? 2 : 1); ++dz)
+#pragma unroll
+      for (int dy = 0; dy < 2; ++dy) {
+        const int k = DIM == 3 ? 2 * K + dz : 0, j = 2 * J + dy, i = 2 * I;
+        const int g = (k * F.n1 + j) * F.n0 + i;
+        Cells<2> X;
+        const Cells<2> r = residual<DIM, 2>(F, F.d + of, F.x + of, ld<2>(F.b + of + g), g, i, j, k, X);
+        acc += r.v[0] + r.v[1];
+      }
+    C.b[oc + t] = acc;
+    C.x2[oc + t] = C.w[oc + t] * acc;
+  });
+}
+
+// The levels of at most kSmallCells cells, of one problem in one CTA: the
+// whole V-cycle from the right-hand side b of the first of them, in shared
+// memory, the result added to its children in xf.
+constexpr int kSmallCells = 512;
+constexpr int kMaxSmall = 6;
+struct SmallLevels {
+  int n, dim, sweeps;                  // levels; sweeps of the coarsest
+  LevDev lev[kMaxSmall];
+  double* xf;
+};
+static size_t small_smem(const SmallLevels& S) {
+  size_t t = 0;
+  for (int l = 0; l < S.n; ++l) t += (size_t)S.lev[l].N * 8;
+  return t * sizeof(double);
+}
+struct SmallLev {
+  double *x, *t, *b, *d, *w, *cx, *cy, *cz;
+};
+__device__ __forceinline__ double small_res(const LevDev& L, const SmallLev& s, const double* x, int g, bool dim3_) {
+  const int sy = L.n0, sz = L.n0 * L.n1;
+  const int k = g / sz, rem = g - k * sz, j = rem / L.n0, i = rem - j * L.n0;
+  double r = s.b[g] - s.d[g] * x[g];
+  if (i > 0) r += s.cx[g - 1] * x[g - 1];
+  if (i < L.n0 - 1) r += s.cx[g] * x[g + 1];
+  if (j > 0) r += s.cy[g - sy] * x[g - sy];
+  if (j < L.n1 - 1) r += s.cy[g] * x[g + sy];
+  if (dim3_) {
+    if (k > 0) r += s.cz[g - sz] * x[g - sz];
+    if (k < L.n2 - 1) r += s.cz[g] * x[g + sz];
+  }
+  return r;
+}
+__global__ void __launch_bounds__(kThreads) mg_small(const __grid_constant__ SmallLevels S, PCGWork w) {
+  extern __shared__ __align__(16) double sm[];
+  if (w.scal[8 * blockIdx.x + 5] != 0.0) return;
+  const bool d3 = S.dim == 3;
+  const int tid = threadIdx.x;
+  SmallLev sl[kMaxSmall];
+  {
+    double* p = sm;
+#pragma unroll
+    for (int l = 0; l < kMaxSmall; ++l) {
+      if (l >= S.n) break;
+      const LevDev& L = S.lev[l];
+      const long long o = (long long)blockIdx.x * L.N;
+      sl[l] = SmallLev{p, p + L.N, p + 2 * L.N, p + 3 * L.N, p + 4 * L.N, p + 5 * L.N, p + 6 * L.N, p + 7 * L.N};
+      p += 8 * L.N;
+      for (int g = tid; g < L.N; g += kThreads) {
+        if (l == 0) sl[l].b[g] = L.b[o + g];
+        sl[l].d[g] = L.d[o + g];
+        sl[l].w[g] = L.w[o + g];
+        sl[l].cx[g] = L.cx[g];
+        sl[l].cy[g] = L.cy[g];
+        if (d3) sl[l].cz[g] = L.cz[g];
+      }
+    }
+  }
+  __syncthreads();
+  auto sweep = [&](int l, const double* in, double* out) {
+    const LevDev& L = S.lev[l];
+    for (int g = tid; g < L.N; g += kThreads) out[g] = in[g] + sl[l].w[g] * small_res(L, sl[l], in, g, d3);
+    __syncthreads();
+  };
+#pragma unroll
+  for (int l = 0; l < kMaxSmall; ++l) {
+    if (l >= S.n) break;
+    const LevDev& L = S.lev[l];
+    double* first = l + 1 < S.n ? sl[l].t : sl[l].x;
+    for (int g = tid; g < L.N; g += kThreads) first[g] = sl[l].w[g] * sl[l].b[g];
+    __syncthreads();
+    if (l + 1 == S.n) {
+      for (int q = 1; q < S.sweeps; q += 2) {                    // (an odd number: the result ends in x)
+        sweep(l, sl[l].x, sl[l].t);
+        sweep(l, sl[l].t, sl[l].x);
+      }
+      break;
+    }
+    sweep(l, sl[l].t, sl[l].x);
+    const LevDev& C = S.lev[l + 1];
+    for (int t = tid; t < C.N; t += kThreads) {
+      const int K = t / (C.n0 * C.n1), rem = t - K * C.n0 * C.n1, J = rem / C.n0, I = rem - J * C.n0;
+      double acc = 0.0;
+      for (int dz = 0; dz < (d3 ? 2 : 1); ++dz)
+        for (int dy = 0; dy < 2; ++dy)
+          for (int dx = 0; dx < 2; ++dx)
+            acc += small_res(L, sl[l], sl[l].x, ((d3 ? 2 * K + dz : 0) * L.n1 + 2 * J + dy) * L.n0 + 2 * I + dx, d3);
+      sl[l + 1].b[t] = acc;
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int l = kMaxSmall - 2; l >= 0; --l) {
+    if (l + 1 >= S.n) continue;
+    const LevDev &L = S.lev[l], &C = S.lev[l + 1];
+    for (int g = tid; g < L.N; g += kThreads) {
+      const int k = g / (L.n0 * L.n1), rem = g - k * L.n0 * L.n1, j = rem / L.n0, i = rem - j * L.n0;
+      sl[l].x[g] += sl[l + 1].x[((d3 ? k >> 1 : 0) * C.n1 + (j >> 1)) * C.n0 + (i >> 1)];
+    }
+    __syncthreads();
+    sweep(l, sl[l].x, sl[l].t);
+    sweep(l, sl[l].t, sl[l].x);
+  }
+  const LevDev& L = S.lev[0];
+  const int f0 = 2 * L.n0, f1 = 2 * L.n1, Nf = L.N * (d3 ? 8 : 4);
+  double* f = S.xf + (long long)blockIdx.x * Nf;
+  for (int g = tid; g < Nf; g += kThreads) {
+    const int k = g / (f0 * f1), rem = g - k * f0 * f1, j = rem / f0, i = rem - j * f0;
+    f[g] += sl[0].x[((d3 ? k >> 1 : 0) * L.n1 + (j >> 1)) * L.n0 + (i >> 1)];
+  }
+}
+
+// All sweeps of a coarsest level above kSmallCells (a grid whose extents turn
+// odd early): eight CTAs of one cluster per problem, a cluster barrier between
+// sweeps (a launch per sweep took 41 launches), the result added to its
+// children in xf.
+constexpr int kClusterCells = 8192, kCoarseCluster = 8, kCoarseThreads = 512;
+__device__ __forceinline__ void coarse_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__global__ void __cluster_dims__(kCoarseCluster, 1, 1) __launch_bounds__(kCoarseThreads)
+mg_coarse_cluster(LevDev L, double* xf, PCGWork w, int dim, int sweeps) {
+  const int b = blockIdx.x / kCoarseCluster;
+  if (w.scal[8 * b + 5] != 0.0) return;                          // (the whole cluster: one problem)
+  const long long o = (long long)b * L.N;
+  const int per = (L.N + kCoarseCluster - 1) / kCoarseCluster;
+  const int g0 = (blockIdx.x % kCoarseCluster) * per, g1 = min(L.N, g0 + per);
+  const int sy = L.n0, sz = L.n0 * L.n1;
+  double *cur = L.x2 + o, *nxt = L.x + o;                        // x2 = w b is there already
+  for (int q = 1; q < sweeps; ++q) {
+    for (int g = g0 + threadIdx.x; g < g1; g += kCoarseThreads) {
+      const int k = g / sz, rem = g - k * sz, j = rem / L.n0, i = rem - j * L.n0;
+      const double x = __ldcg(cur + g);
+      double r = L.b[o + g] - L.d[o + g] * x;
+      if (i > 0) r += L.cx[g - 1] * __ldcg(cur + g - 1);
+      if (i < L.n0 - 1) r += L.cx[g] * __ldcg(cur + g + 1);
+      if (j > 0) r += L.cy[g - sy] * __ldcg(cur + g - sy);
+      if (j < L.n1 - 1) r += L.cy[g] * __ldcg(cur + g + sy);
+      if (dim == 3) {
+        if (k > 0) r += L.cz[g - sz] * __ldcg(cur + g - sz);
+        if (k < L.n2 - 1) r += L.cz[g] * __ldcg(cur + g + sz);
+      }
+      nxt[g] = x + L.w[o + g] * r;
+    }
+    coarse_sync();
     double* t = cur;
     cur = nxt;
     nxt = t;
   }
-  __syncthreads();
-  if (cur != x + o)
-    for (int g = threadIdx.x; g < a.N; g += blockDim.x) x[o + g] = cur[g];
-}
-
-static dim3 mg_grid(int N, int batch) {
-  return dim3((unsigned)std::min(kPCGBlocks, (N + kThreads - 1) / kThreads), batch);
-}
-
-// z = V-cycle(r) for level l; x/x2/b of level 0 are bound by the caller.
-static void mg_vcycle(MGHierarchy& h, int l, int batch, cudaStream_t s) {
-  MGLevel& L = h.lev[l];
-  const dim3 g = mg_grid(L.A.N, batch);
-  if (l == h.nlev - 1 && L.A.N <= kCoarseCells) {
-    mg_coarse_kernel<<<batch, 1024, 0, s>>>(L.A, L.mu, L.b, L.x, L.x2, h.omega, h.coarse_sweeps);
-    return;
-  }
-  if (l == h.nlev - 1) {
-    mg_jacobi_kernel<<<g, kThreads, 0, s>>>(L.A, L.mu, L.x, L.b, L.x, h.omega, 1);
-    for (int it = 1; it < h.coarse_sweeps; ++it) {
-      mg_jacobi_kernel<<<g, kThreads, 0, s>>>(L.A, L.mu, L.x, L.b, L.x2, h.omega, 0);
-      mg_jacobi_kernel<<<g, kThreads, 0, s>>>(L.A, L.mu, L.x2, L.b, L.x, h.omega, 0);
-      ++it;
+  const int f0 = 2 * L.n0, f1 = 2 * L.n1, nch = dim == 3 ? 4 : 2;
+  double* f = xf + (long long)b * L.N * (dim == 3 ? 8 : 4);
+  for (int g = g0 + threadIdx.x; g < g1; g += kCoarseThreads) {
+    const int k = g / sz, rem = g - k * sz, j = rem / L.n0, i = rem - j * L.n0;
+    const double v = __ldcg(cur + g);
+    for (int q = 0; q < nch; ++q) {
+      double* p = f + ((long long)(dim == 3 ? 2 * k + (q >> 1) : 0) * f1 + 2 * j + (q & 1)) * f0 + 2 * i;
+      p[0] += v;
+      p[1] += v;
     }
-    return;
   }
-  MGLevel& Cl = h.lev[l + 1];
-  // pre-smoothing: nu sweeps from zero, result in x
-  mg_jacobi_kernel<<<g, kThreads, 0, s>>>(L.A, L.mu, L.x, L.b, L.x2, h.omega, 1);
-  mg_jacobi_kernel<<<g, kThreads, 0, s>>>(L.A, L.mu, L.x2, L.b, L.x, h.omega, 0);
-  mg_restrict_kernel<<<mg_grid(Cl.A.N, batch), kThreads, 0, s>>>(L.A, L.mu, L.x, L.b, Cl.b, Cl.A.n0, Cl.A.n1, Cl.A.n2);
-  mg_vcycle(h, l + 1, batch, s);
-  mg_prolong_kernel<<<g, kThreads, 0, s>>>(L.A, Cl.x, L.x, Cl.A.n0, Cl.A.n1, Cl.A.n2);
-  // post-smoothing: the same nu sweeps, result in x
-  mg_jacobi_kernel<<<g, kThreads, 0, s>>>(L.A, L.mu, L.x, L.b, L.x2, h.omega, 0);
-  mg_jacobi_kernel<<<g, kThreads, 0, s>>>(L.A, L.mu, L.x2, L.b, L.x, h.omega, 0);
 }
 
-__global__ void pcg_init_mg_kernel(DAArgs a, const double* rhs, PCGWork w) {
-  const int b = blockIdx.y;
-  const long long o = (long long)b * a.N;
-  double rr = 0;
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.N; g += gridDim.x * blockDim.x) {
-    const double r = rhs[o + g];
-    w.x[o + g] = 0.0;
-    w.r[o + g] = r;
-    rr += r * r;
-  }
-  block_sum3(0.0, rr, rr, w.partial + ((long long)b * kPCGBlocks + blockIdx.x) * 4);
+// First level (at least 1) from which all levels fit mg_small; nlev if none.
+static int small_from(const MGHierarchy& h) {
+  int l = h.nlev;
+  size_t cells = 0;
+  while (l > 1 && h.lev[l - 1].A.N <= kSmallCells && h.nlev - l < kMaxSmall) cells += h.lev[--l].A.N;
+  return l;
 }
 
-// x += alpha p, r -= alpha q, partial r.r  (the preconditioner runs after)
-__global__ void pcg_update_mg_kernel(DAArgs a, PCGWork w, int parity) {
-  const int b = blockIdx.y;
-  const long long o = (long long)b * a.N;
-  const double* sc = w.scal + 8 * b;
-  const bool done = sc[5] != 0.0;
+// z = V-cycle(r): r.z goes to scal[slot].  Level 0's x2 = w r is there already.
+static void mg_vcycle(MGHierarchy& h, PCGWork& w, int batch, int slot, cudaStream_t s) {
+  const int ls = small_from(h), dim = h.lev[0].A.dim;
+  const int bottom = ls < h.nlev ? ls : h.nlev - 1;              // first level not smoothed by launches of its own
+  for (int l = 0; l < bottom; ++l) {
+    const LevDev L = mg_dev(h.lev[l], w), C = mg_dev(h.lev[l + 1], w);
+    const MGGrid g = mg_grid(h.lev[l].A, batch);
+    MG_DISPATCH(h.lev[l].A, mg_sweep, g, s, L, L.x2, L.x, w);
+    MGGrid gc = mg_grid(h.lev[l + 1].A, batch);
+    if (dim == 3) mg_restrict<3><<<gc.grid, gc.block, 0, s>>>(L, C, w);
+    else mg_restrict<2><<<gc.grid, gc.block, 0, s>>>(L, C, w);
+  }
+  const MGLevel& B = h.lev[bottom];
+  double* xf = h.lev[bottom - 1].x;
+  if (ls < h.nlev) {
+    SmallLevels S{};
+    S.n = h.nlev - ls;
+    S.dim = dim;
+    S.sweeps = h.coarse_sweeps;
+    for (int l = ls; l < h.nlev; ++l) S.lev[l - ls] = mg_dev(h.lev[l], w);
+    S.xf = xf;
+    mg_small<<<batch, kThreads, small_smem(S), s>>>(S, w);
+  } else if (B.A.N <= kClusterCells) {
+    mg_coarse_cluster<<<kCoarseCluster * batch, kCoarseThreads, 0, s>>>(mg_dev(B, w), xf, w, dim, h.coarse_sweeps);
+  } else {
+    const LevDev L = mg_dev(B, w);
+    const MGGrid g = mg_grid(B.A, batch);
+    double *cur = L.x2, *nxt = L.x;
+    for (int it = 1; it + 1 < h.coarse_sweeps; ++it) {
+      MG_DISPATCH(B.A, mg_sweep, g, s, L, cur, nxt, w);
+      std::swap(cur, nxt);
+    }
+    MG_DISPATCH(B.A, mg_sweep_prolong, g, s, L, cur, xf, w);
+  }
+  for (int l = bottom - 1; l >= 0; --l) {
+    const LevDev L = mg_dev(h.lev[l], w);
+    const MGGrid g = mg_grid(h.lev[l].A, batch);
+    MG_DISPATCH(h.lev[l].A, mg_sweep, g, s, L, L.x, L.x2, w);
+    if (l == 0) MG_DISPATCH(h.lev[l].A, mg_sweep_dot, g, s, L, L.x2, L.x, w, slot);
+    else MG_DISPATCH(h.lev[l].A, mg_sweep_prolong, g, s, L, L.x2, h.lev[l - 1].x, w);
+  }
+}
+
+// The vectors of one problem as [0, N) in pairs of cells: body(t) for t = 0, 2, ...
+template <class F>
+__device__ __forceinline__ void for_pairs(int N, F&& body) {
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  for (int t = 2 * (blockIdx.x * kThreads + tid); t < N; t += 2 * (int)gridDim.x * kThreads) body(t);
+}
+
+// x = 0, r = rhs, the first sweep of the V-cycle, bb = rr = rhs.rhs
+__global__ void __launch_bounds__(kThreads) pcg_init_mg(int N, const double* rhs, PCGWork w) {
+  const long long o = (long long)blockIdx.y * N;
+  double *x = w.x + o, *r = w.r + o, *x2 = w.mg_x2 + o;
+  const double *q = rhs + o, *wd = w.dinv + o;
+  double rr = 0.0;
+  for_pairs(N, [&](int t) {                                      // (N is even: mg needs even extents)
+    const Cells<2> v = ld<2>(q + t), m = ld<2>(wd + t);
+    st<2>(x + t, Cells<2>{{0.0, 0.0}});
+    st<2>(r + t, v);
+    st<2>(x2 + t, Cells<2>{{m.v[0] * v.v[0], m.v[1] * v.v[1]}});
+    rr += v.v[0] * v.v[0] + v.v[1] * v.v[1];
+  });
+  if (last_block_sum(rr, w)) {
+    w.scal[8 * blockIdx.y + 3] = rr;
+    w.scal[8 * blockIdx.y + 4] = rr;
+  }
+}
+
+// q = A p, p.q
+template <int DIM, int VEC>
+__global__ void __launch_bounds__(kThreads) pcg_spmv_mg(LevDev L, PCGWork w) {
+  if (pcg_done(w)) return;
+  const long long o = (long long)blockIdx.y * L.N;
+  double pq = 0.0;
+  for_groups<DIM, VEC>(L.n0, L.n1, L.n2, [&](int g, int i, int j, int k) {
+    Cells<VEC> X, r;
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) r.v[v] = 0.0;
+    r = residual<DIM, VEC>(L, L.d + o, w.p + o, r, g, i, j, k, X);
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) {
+      r.v[v] = -r.v[v];
+      pq += X.v[v] * r.v[v];
+    }
+    st<VEC>(w.q + o + g, r);
+  });
+  if (last_block_sum(pq, w)) w.scal[8 * blockIdx.y + 2] = pq;
+}
+
+// x += alpha p, r -= alpha q, the first sweep of the V-cycle on r, r.r, and the
+// convergence flag
+__global__ void __launch_bounds__(kThreads) pcg_update_mg(int N, PCGWork w, int parity, double tol2) {
+  double* sc = w.scal + 8 * blockIdx.y;
+  if (sc[5] != 0.0) return;
+  const long long o = (long long)blockIdx.y * N;
+  double *x = w.x + o, *r = w.r + o, *x2 = w.mg_x2 + o;
+  const double *p = w.p + o, *q = w.q + o, *wd = w.dinv + o;
   const double rz = sc[parity], pq = sc[2];
-  const double alpha = (done || pq == 0.0) ? 0.0 : rz / pq;
-  double rr = 0;
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.N; g += gridDim.x * blockDim.x) {
-    w.x[o + g] += alpha * w.p[o + g];
-    const double r = w.r[o + g] - alpha * w.q[o + g];
-    w.r[o + g] = r;
-    rr += r * r;
+  const double alpha = pq == 0.0 ? 0.0 : rz / pq;
+  double rr = 0.0;
+  for_pairs(N, [&](int t) {
+    Cells<2> X = ld<2>(x + t), R = ld<2>(r + t), M = ld<2>(wd + t);
+    const Cells<2> P = ld<2>(p + t), Q = ld<2>(q + t);
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      X.v[v] += alpha * P.v[v];
+      R.v[v] -= alpha * Q.v[v];
+      M.v[v] *= R.v[v];
+      rr += R.v[v] * R.v[v];
+    }
+    st<2>(x + t, X);
+    st<2>(r + t, R);
+    st<2>(x2 + t, M);
+  });
+  if (last_block_sum(rr, w)) {
+    sc[3] = rr;
+    if (rr <= tol2 * sc[4]) sc[5] = 1.0;
   }
-  block_sum3(0.0, rr, 0.0, w.partial + ((long long)b * kPCGBlocks + blockIdx.x) * 4);
 }
 
-__global__ void pcg_dot_rz_kernel(DAArgs a, PCGWork w, int set_p) {
-  const int b = blockIdx.y;
-  const long long o = (long long)b * a.N;
-  double rz = 0;
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.N; g += gridDim.x * blockDim.x) {
-    rz += w.r[o + g] * w.z[o + g];
-    if (set_p) w.p[o + g] = w.z[o + g];
-  }
-  block_sum3(rz, 0.0, 0.0, w.partial + ((long long)b * kPCGBlocks + blockIdx.x) * 4);
+// p = z + beta p (first: p = z)
+__global__ void __launch_bounds__(kThreads) pcg_pupdate_mg(int N, PCGWork w, int parity, int first) {
+  const double* sc = w.scal + 8 * blockIdx.y;
+  if (sc[5] != 0.0) return;
+  const long long o = (long long)blockIdx.y * N;
+  double* p = w.p + o;
+  const double* z = w.z + o;
+  const double rz_old = sc[parity], rz_new = sc[parity ^ 1];
+  const double beta = (first || rz_old == 0.0) ? 0.0 : rz_new / rz_old;
+  for_pairs(N, [&](int t) {
+    Cells<2> Z = ld<2>(z + t);
+    if (!first) {
+      const Cells<2> P = ld<2>(p + t);
+#pragma unroll
+      for (int v = 0; v < 2; ++v) Z.v[v] += beta * P.v[v];
+    }
+    st<2>(p + t, Z);
+  });
 }
 
 // One conjugate-gradient iteration of every problem in the batch (parity =
 // iteration number mod 2 selects the slot holding the current r.z).
-static void pcg_iteration(const DAArgs& a, const double* mu, int batch, PCGWork& w, int parity, cudaStream_t s) {
-  const dim3 grid(kPCGBlocks, batch);
+static void pcg_iteration(const DAArgs& a, const double* mu, int batch, PCGWork& w, int parity, double tol2,
+                          cudaStream_t s) {
   MGHierarchy* mg = w.mg;
+  if (mg && mg->nlev > 0) {
+    const MGGrid g = mg_grid(a, batch);
+    MG_DISPATCH(a, pcg_spmv_mg, g, s, mg_dev(mg->lev[0], w), w);
+    pcg_update_mg<<<g.grid, g.block, 0, s>>>(a.N, w, parity, tol2);
+    mg_vcycle(*mg, w, batch, parity ^ 1, s);
+    pcg_pupdate_mg<<<g.grid, g.block, 0, s>>>(a.N, w, parity, 0);
+    return;
+  }
+  const dim3 grid(kPCGBlocks, batch);
   pcg_spmv_kernel<<<grid, kThreads, 0, s>>>(a, mu, w);
   pcg_reduce_kernel<<<batch, kThreads, 0, s>>>(w, 2, -1, -1);
-  if (mg && mg->nlev > 0) {
-    pcg_update_mg_kernel<<<grid, kThreads, 0, s>>>(a, w, parity);
-    pcg_reduce_kernel<<<batch, kThreads, 0, s>>>(w, -1, 3, -1);
-    mg_vcycle(*mg, 0, batch, s);
-    pcg_dot_rz_kernel<<<grid, kThreads, 0, s>>>(a, w, 0);
-    pcg_reduce_kernel<<<batch, kThreads, 0, s>>>(w, parity ^ 1, -1, -1);
-  } else {
-    pcg_update_kernel<<<grid, kThreads, 0, s>>>(a, w, parity);
-    pcg_reduce_kernel<<<batch, kThreads, 0, s>>>(w, parity ^ 1, 3, -1);
-  }
+  pcg_update_kernel<<<grid, kThreads, 0, s>>>(a, w, parity);
+  pcg_reduce_kernel<<<batch, kThreads, 0, s>>>(w, parity ^ 1, 3, -1);
   pcg_pupdate_kernel<<<grid, kThreads, 0, s>>>(a, w, parity);
+  pcg_mark_done_kernel<<<(batch + 127) / 128, 128, 0, s>>>(w, batch, tol2);
 }
 
 int pcg_solve(const DAArgs& a, const double* mu_in, int batch, const double* rhs, double* x, PCGWork& w,
@@ -473,29 +917,33 @@ int pcg_solve(const DAArgs& a, const double* mu_in, int batch, const double* rhs
   const double tol2 = tol * tol;
   MGHierarchy* mg = w.mg;
   const bool multigrid = mg && mg->nlev > 0;
-  // the iterations read mu from a buffer of their own, so that a captured
-  // chunk of them stays valid for every call
-  copy_kernel<<<256, kThreads, 0, s>>>((long long)batch * a.N, mu_in, w.mu);
-  const double* mu = w.mu;
   cudaMemsetAsync(w.scal, 0, sizeof(double) * 8 * batch, s);
+  const double* mu = w.mu;
   if (multigrid) {
-    // level 0 of the hierarchy works on the PCG vectors: the V-cycle maps r to z
+    // level 0 of the hierarchy works on the PCG vectors (the V-cycle maps r to
+    // z); the iterations read the levels' diagonals, built here from mu, so
+    // that a captured chunk of them stays valid for every call
     MGLevel& L0 = mg->lev[0];
     L0.A = a;
-    L0.mu = w.mu;
+    L0.d = w.b;
+    L0.w = w.dinv;
     L0.b = w.r;
     L0.x = w.z;
+    w.mg_x2 = L0.x2;
+    mg_diag_kernel<<<mg_blocks(a.N, batch), kThreads, 0, s>>>(a, mu_in, mg->omega, L0.d, L0.w);
+    const double* muf = mu_in;
     for (int l = 1; l < mg->nlev; ++l) {
       const DAArgs& f = mg->lev[l - 1].A;
-      coarsen_mean_kernel<<<dim3(128, batch), kThreads, 0, s>>>(mg->lev[l - 1].mu, mg->lev[l].mu, f.n0, f.n1, f.n2,
-                                                                 f.dim, f.N, mg->lev[l].A.N);
+      MGLevel& L = mg->lev[l];
+      mg_coarsen_kernel<<<mg_blocks(L.A.N, batch), kThreads, 0, s>>>(f, L.A, muf, mg->omega, L.mu, L.d, L.w);
+      muf = L.mu;
     }
-    pcg_init_mg_kernel<<<grid, kThreads, 0, s>>>(a, rhs, w);
-    pcg_reduce_kernel<<<batch, kThreads, 0, s>>>(w, -1, 3, 4);
-    mg_vcycle(*mg, 0, batch, s);
-    pcg_dot_rz_kernel<<<grid, kThreads, 0, s>>>(a, w, 1);
-    pcg_reduce_kernel<<<batch, kThreads, 0, s>>>(w, 0, -1, -1);
+    const MGGrid g = mg_grid(a, batch);
+    pcg_init_mg<<<g.grid, g.block, 0, s>>>(a.N, rhs, w);
+    mg_vcycle(*mg, w, batch, 0, s);
+    pcg_pupdate_mg<<<g.grid, g.block, 0, s>>>(a.N, w, 0, 1);
   } else {
+    copy_kernel<<<256, kThreads, 0, s>>>((long long)batch * a.N, mu_in, w.mu);
     pcg_init_kernel<<<grid, kThreads, 0, s>>>(a, mu, rhs, w);
     pcg_reduce_kernel<<<batch, kThreads, 0, s>>>(w, 0, 3, 4);
   }
@@ -511,8 +959,7 @@ int pcg_solve(const DAArgs& a, const double* mu_in, int batch, const double* rhs
     if (!w.cap && (*err = cudaStreamCreateWithFlags(&w.cap, cudaStreamNonBlocking)) != cudaSuccess) return -1;
     if ((*err = cudaStreamBeginCapture(w.cap, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return -1;
     for (int k = 0; k < chunk; ++k) {
-      pcg_iteration(a, mu, batch, w, k & 1, w.cap);
-      pcg_mark_done_kernel<<<(batch + 127) / 128, 128, 0, w.cap>>>(w, batch, tol2);
+      pcg_iteration(a, mu, batch, w, k & 1, tol2, w.cap);
     }
     cudaGraph_t g = nullptr;
     *err = cudaStreamEndCapture(w.cap, &g);
@@ -530,8 +977,7 @@ int pcg_solve(const DAArgs& a, const double* mu_in, int batch, const double* rhs
       if ((*err = cudaGraphLaunch(w.chunk, s)) != cudaSuccess) return -1;
     } else {
       for (int k = 0; k < len; ++k) {
-        pcg_iteration(a, mu, batch, w, k & 1, s);
-        pcg_mark_done_kernel<<<(batch + 127) / 128, 128, 0, s>>>(w, batch, tol2);
+        pcg_iteration(a, mu, batch, w, k & 1, tol2, s);
       }
     }
     it += len;

@@ -171,6 +171,7 @@ cudaError_t da_setup(DAArgs& a, double* d_diag0, double* d_cxf, double* d_cyf, d
 struct MGLevel {
   DAArgs A;
   double *mu, *x, *x2, *b;
+  double *d, *w;           // diagonal of A and omega / d for the absorption of the current solve
   double* kappa;           // the level's kappa (the fine level: the context's)
 };
 constexpr int kMaxLevels = 16;
@@ -184,7 +185,9 @@ struct MGHierarchy {
 
 struct PCGWork {
   double *x, *r, *z, *p, *q, *dinv, *b;   // [B][N]
-  double *partial;                         // [B][kPartials][4]
+  double *partial;                         // [B][kPCGBlocks][4]
+  double* mg_x2;                           // level-0 scratch of the V-cycle
+  unsigned* count;                         // [B] blocks done, of the reductions that finish in the last block
   double *scal;                            // [B][8]
   double *hostscal;                        // pinned [B][8]
   MGHierarchy* mg;                         // null: Jacobi preconditioner
