@@ -141,11 +141,36 @@ cudaError_t dalloc(qpat_ctx* c, P** p, size_t bytes) {
 
 cudaError_t dalloc_cb(void* owner, void** p, size_t bytes) { return dalloc((qpat_ctx*)owner, p, bytes); }
 
-// Radices of an extent, fewest stages first: 8s, then what is left of the
-// twos (a single one joins a three as radix 6), pairs of threes as 9.
-bool factor_plan(int L, FFTPlan& p) {
-  p.L = L;
-  p.nstages = 0;
+// FP64 radices of an extent: the factorisation into 2, 3, 4, 5, 7, 8 with the
+// least work, where a stage of radix R costs its warps of butterflies for two lines
+// (what a CTA of the smallest launches transforms; a half-empty warp holds the
+// two FP64 lanes of its SM as long as a full one) times the FP64 instructions
+// of one butterfly, and a barrier.  Fewest stages would take 48 as 8 6, sixteen
+// lanes of a warp: 60 x 48, 400 steps, forward + adjoint 65.2 ms, against 55.0
+// ms as 4 4 3.
+void search_plan(int L, int rest, int most, double cost, const int* now, int n, double& best, FFTPlan& p) {
+  static const double work[9] = {0, 0, 8, 24, 28, 56, 0, 96, 92};
+  if (cost >= best) return;
+  if (rest == 1) {
+    best = cost;
+    p.nstages = n;
+    for (int k = 0; k < n; ++k) p.radix[k] = now[k];
+    return;
+  }
+  if (n == kMaxStages) return;
+  int next[kMaxStages];
+  for (int k = 0; k < n; ++k) next[k] = now[k];
+  for (int q = std::min(most, 8); q >= 2; --q) {
+    if (rest % q || q == 6) continue;
+    next[n] = q;
+    search_plan(L, rest / q, q, cost + (2 * L / q + 31) / 32 * work[q] + 25.0, next, n + 1, best, p);
+  }
+}
+
+// FP32 radices: fewest stages (the index arithmetic of a stage outweighs its
+// FP32 work): 8s, then what is left of the twos (a single one joins a three as
+// radix 6), pairs of threes as 9.
+bool short_plan(int L, FFTPlan& p) {
   int r = L;
   int twos = 0, threes = 0;
   while (r % 2 == 0) { r /= 2; ++twos; }
@@ -169,6 +194,16 @@ bool factor_plan(int L, FFTPlan& p) {
     }
   }
   return ok && r == 1;
+}
+
+bool factor_plan(int L, FFTPlan& p, int elt) {
+  p.L = L;
+  p.nstages = 0;
+  if (elt == 4) return short_plan(L, p);
+  double best = 1e300;
+  const int none[kMaxStages] = {};
+  search_plan(L, L, 8, 0.0, none, 0, best, p);
+  return best < 1e300;
 }
 
 template <typename T>
@@ -270,7 +305,8 @@ qpat_status build_context3(qpat_ctx* c, const qpat_medium* med, const double* se
   Prop3<T>& a = args3<T>(c);
   a.nx = c->nx; a.ny = c->ny; a.nz = c->nz; a.nxh = c->nxh; a.pitch = c->pitch; a.pml = c->pml;
   a.n0 = c->n0; a.n1 = c->n1; a.n2 = c->n2; a.ns = c->ns; a.nt = c->nt;
-  if (!factor_plan(c->nx, a.px) || !factor_plan(c->ny, a.py) || !factor_plan(c->nz, a.pz))
+  if (!factor_plan(c->nx, a.px, (int)sizeof(T)) || !factor_plan(c->ny, a.py, (int)sizeof(T)) ||
+      !factor_plan(c->nz, a.pz, (int)sizeof(T)))
     return fail(c, QPAT_EINVAL, "FFT extents must factor into 2, 3, 5 and 7");
   a.cby = a.cbz = 1;
   for (int cb : {8, 4, 2}) {
@@ -352,7 +388,7 @@ qpat_status build_context(qpat_ctx* c, const qpat_medium* med, const double* sen
   PropArgs<T>& a = args<T>(c);
   a.nx = c->nx; a.ny = c->ny; a.nxh = c->nxh; a.pitch = c->pitch; a.pml = c->pml;
   a.n0 = c->n0; a.n1 = c->n1; a.ns = c->ns; a.nt = c->nt;
-  if (!factor_plan(c->nx, a.px) || !factor_plan(c->ny, a.py))
+  if (!factor_plan(c->nx, a.px, (int)sizeof(T)) || !factor_plan(c->ny, a.py, (int)sizeof(T)))
     return fail(c, QPAT_EINVAL, "FFT extents must factor into 2, 3, 5 and 7");
   // column tile width: widest of 8/4/2/1 columns whose tile fits 100 KB of shared memory
   a.cb = 1;

@@ -229,6 +229,9 @@ __device__ __forceinline__ void stockham_stage(const C* __restrict__ in, C* __re
 // Must be called by all threads of the CTA; ends with __syncthreads().
 template <typename C>
 __device__ C* fft_batch(const FFTPlan& plan, C* buf0, C* buf1, int M, int S, const C* __restrict__ tw) {
+  // radices 6 and 9 only in FP32: in FP64 their registers (126 a thread) halve
+  // the resident CTAs of every pass, and plans have none
+  constexpr bool kWide = sizeof(C) == 8;
   C* in = buf0;
   C* out = buf1;
   int Ns = 1;
@@ -239,10 +242,10 @@ __device__ C* fft_batch(const FFTPlan& plan, C* buf0, C* buf1, int M, int S, con
       case 3: stockham_stage<3>(in, out, plan.L, M, S, Ns, tw); break;
       case 4: stockham_stage<4>(in, out, plan.L, M, S, Ns, tw); break;
       case 5: stockham_stage<5>(in, out, plan.L, M, S, Ns, tw); break;
-      case 6: stockham_stage<6>(in, out, plan.L, M, S, Ns, tw); break;
+      case 6: if constexpr (kWide) stockham_stage<6>(in, out, plan.L, M, S, Ns, tw); break;
       case 7: stockham_stage<7>(in, out, plan.L, M, S, Ns, tw); break;
       case 8: stockham_stage<8>(in, out, plan.L, M, S, Ns, tw); break;
-      case 9: stockham_stage<9>(in, out, plan.L, M, S, Ns, tw); break;
+      case 9: if constexpr (kWide) stockham_stage<9>(in, out, plan.L, M, S, Ns, tw); break;
       default: break;
     }
     __syncthreads();

@@ -44,12 +44,6 @@ template <> struct ColIO<A_C6> { static constexpr int kin = 2, kout = 1; };
 
 constexpr int kRowThreads = 256;
 constexpr int kColThreads = 256;
-// Resident CTAs per SM the generic passes are compiled for: the radix-9
-// butterfly would otherwise take 56-64 registers a thread in FP32 (126 in
-// FP64) in every launch, also where no stage uses it.
-template <typename T>
-constexpr int generic_minb() { return sizeof(T) == 4 ? 5 : 3; }
-
 template <typename T>
 size_t row_smem_bytes(int nx) {
   typedef typename V2<T>::t C;

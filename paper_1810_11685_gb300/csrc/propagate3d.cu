@@ -24,7 +24,7 @@ namespace qpat {
 
 // ---- x row pass: rows (k, j0) and (k, j0+1) of problem blockIdx.z ----------
 template <typename T, int PH>
-__global__ void __launch_bounds__(k3Threads) row3_kernel(const Prop3<T> a) {
+__global__ void __launch_bounds__(k3Threads, generic_minb<T>()) row3_kernel(const Prop3<T> a) {
   typedef typename V2<T>::t C;
   constexpr int KIN = r3_kin(PH), KOUT = r3_kout(PH);
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(k3Threads) row3_kernel(const Prop3<T> a) {
 
 // ---- y pass: forward (INV = 0) or inverse (INV = 1) y-FFT of K slots -------
 template <typename T, int K, int INV>
-__global__ void __launch_bounds__(k3Threads) ypass3_kernel(const Prop3<T> a, const int gather) {
+__global__ void __launch_bounds__(k3Threads, generic_minb<T>()) ypass3_kernel(const Prop3<T> a, const int gather) {
   typedef typename V2<T>::t C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int cb = a.cby, ny = a.ny, S = ny + 1, nxh = a.nxh;
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(k3Threads) ypass3_kernel(const Prop3<T> a, con
 
 // ---- z pass: forward z-FFT, k-space symbol, inverse z-FFT -----------------
 template <typename T, int PH>
-__global__ void __launch_bounds__(k3Threads) zpass3_kernel(const Prop3<T> a) {
+__global__ void __launch_bounds__(k3Threads, generic_minb<T>()) zpass3_kernel(const Prop3<T> a) {
   typedef typename V2<T>::t C;
   constexpr int KIN = z3_kin(PH), KOUT = z3_kout(PH);
   extern __shared__ __align__(16) unsigned char smem_raw[];
