@@ -193,6 +193,8 @@ qpat_status qpat_vjp_kappa(qpat_ctx* ctx, int batch, const double* mu, const dou
  * A checkpoint holds, per problem, v_x, v_y, rho_x, rho_y, the sampling
  * buffer and the two spectral work slots after loop iteration n with
  * (n + 1) % K == 0 (Section 3.2.3 loop), m = (n + 1)/K - 1, 0 <= m < (nt-1)/K.
+ * (The work slots' layout belongs to the kernels the context runs: resume a
+ * checkpoint on the context, and at the batch, that wrote it.)
  * qpat_ckpt_bytes: size of the checkpoint buffer for batch and K.
  * qpat_acoustic_forward_ckpt: H_a as qpat_acoustic_forward, also filling
  *   ckpt (device, caller-owned, qpat_ckpt_bytes bytes).
@@ -305,7 +307,8 @@ qpat_status qpat_group_tune(qpat_group* group, const int* batches, int steps, vo
 /* Autotuner: time a `steps`-step forward + adjoint of `batch` problems with
  * every supported choice of pass kernels (specialised or generic row passes,
  * specialised or generic column passes) and keep the fastest for this
- * context; *choice = bit 0 rows specialised, bit 1 columns specialised.
+ * context; *choice = bit 0 rows specialised, bit 1 columns specialised (3
+ * also for the whole-loop kernel of small 2D FP32 grids).
  * Synchronises; allocates and frees temporary buffers. */
 qpat_status qpat_autotune(qpat_ctx* ctx, int batch, int steps, int* choice);
 

@@ -21,6 +21,7 @@
 #include "qpat_internal.h"
 #include "prop3d.h"
 #include "multi.h"
+#include "loop2d.h"
 
 using namespace qpat;
 
@@ -61,6 +62,8 @@ struct qpat_ctx {
   std::map<int, std::pair<cudaGraphExec_t, long long>> graphs;   // (dir, batch) -> graph, kernels
   std::vector<cudaEvent_t> prof_events;
   size_t prof_used = 0;
+  LoopPlan loop;               // whole-loop kernel of small 2D FP32 grids
+  int loop_on = 0;             // 1: propagations run it
   int medium_k = 0;            // checkpoint interval of the medium gradient (0: automatic)
 };
 
@@ -472,7 +475,7 @@ qpat_status build_context(qpat_ctx* c, const qpat_medium* med, const double* sen
     }
   }
   std::sort(ent.begin(), ent.end());
-  std::vector<int> rowptr(c->ny + 1, 0), pcol, pent, esens;
+  std::vector<int> rowptr(c->ny + 1, 0), pcol, prow, pent, esens;
   std::vector<T> ew;
   {
     int prev_r = -1, prev_c = -1;
@@ -480,6 +483,7 @@ qpat_status build_context(qpat_ctx* c, const qpat_medium* med, const double* sen
       const int r = std::get<0>(ent[e]), col = std::get<1>(ent[e]);
       if (r != prev_r || col != prev_c) {
         pcol.push_back(col);
+        prow.push_back(r);
         pent.push_back((int)e);
         rowptr[r + 1] += 1;
         prev_r = r;
@@ -491,12 +495,13 @@ qpat_status build_context(qpat_ctx* c, const qpat_medium* med, const double* sen
     pent.push_back((int)ent.size());
     for (int r = 0; r < c->ny; ++r) rowptr[r + 1] += rowptr[r];
   }
-  int *d_sidx, *d_rowptr, *d_pcol, *d_pent, *d_esens;
+  int *d_sidx, *d_rowptr, *d_pcol, *d_prow, *d_pent, *d_esens;
   T *d_sw, *d_ew;
   QCK(dalloc(c, &d_sidx, sidx.size() * sizeof(int)));
   QCK(dalloc(c, &d_sw, sw.size() * sizeof(T)));
   QCK(dalloc(c, &d_rowptr, rowptr.size() * sizeof(int)));
   QCK(dalloc(c, &d_pcol, std::max<size_t>(1, pcol.size()) * sizeof(int)));
+  QCK(dalloc(c, &d_prow, std::max<size_t>(1, prow.size()) * sizeof(int)));
   QCK(dalloc(c, &d_pent, pent.size() * sizeof(int)));
   QCK(dalloc(c, &d_esens, std::max<size_t>(1, esens.size()) * sizeof(int)));
   QCK(dalloc(c, &d_ew, std::max<size_t>(1, ew.size()) * sizeof(T)));
@@ -504,10 +509,11 @@ qpat_status build_context(qpat_ctx* c, const qpat_medium* med, const double* sen
   QCK(cudaMemcpy(d_sw, sw.data(), sw.size() * sizeof(T), cudaMemcpyHostToDevice));
   QCK(cudaMemcpy(d_rowptr, rowptr.data(), rowptr.size() * sizeof(int), cudaMemcpyHostToDevice));
   if (!pcol.empty()) QCK(cudaMemcpy(d_pcol, pcol.data(), pcol.size() * sizeof(int), cudaMemcpyHostToDevice));
+  if (!prow.empty()) QCK(cudaMemcpy(d_prow, prow.data(), prow.size() * sizeof(int), cudaMemcpyHostToDevice));
   QCK(cudaMemcpy(d_pent, pent.data(), pent.size() * sizeof(int), cudaMemcpyHostToDevice));
   if (!esens.empty()) QCK(cudaMemcpy(d_esens, esens.data(), esens.size() * sizeof(int), cudaMemcpyHostToDevice));
   if (!ew.empty()) QCK(cudaMemcpy(d_ew, ew.data(), ew.size() * sizeof(T), cudaMemcpyHostToDevice));
-  a.sidx = d_sidx; a.sw = d_sw; a.rowptr = d_rowptr; a.pcol = d_pcol; a.pent = d_pent; a.esens = d_esens; a.ew = d_ew;
+  a.sidx = d_sidx; a.sw = d_sw; a.rowptr = d_rowptr; a.pcol = d_pcol; a.prow = d_prow; a.pent = d_pent; a.esens = d_esens; a.ew = d_ew;
 
   // workspace
   a.gstride = G;
@@ -529,6 +535,11 @@ qpat_status build_context(qpat_ctx* c, const qpat_medium* med, const double* sen
   a.io = io;
   a.err = c->d_err;
   prop_init_attributes<T>(c->nx, c->ny, a.fast_rows, a.fast_cols);
+  if constexpr (std::is_same<T, float>::value) {
+    // (cfg.generic_fft asks for the generic passes)
+    if (!c->cfg.generic_fft) loop_plan(a, c->cfg.lossless, c->maxb, c->c_ref, c->dt, c->cfg.y, &c->loop);
+    c->loop_on = c->loop.ok;
+  }
   return QPAT_OK;
 }
 
@@ -564,6 +575,50 @@ void pass(qpat_ctx* c, const PropArgs<T>& a, int phase, int batch, bool is_row, 
   }
 }
 
+// Whether a propagation of `batch` problems runs the whole-loop kernel: while
+// their clusters are resident at once, and beyond that where square grids of
+// the extent have a kernel of their own and the launched passes no
+// length-specialised form.  (100 steps, forward + adjoint, loop kernel against
+// launched passes, ms: 168^2, specialised passes, 6 problems 4.3 / 6.8, 8
+// 8.6 / 6.9; 200^2 4 5.0 / 9.6, 32 25.1 / 33.3; 216 x 168 4 6.8 / 7.2, 16
+// 20.2 / 13.3.)  The pass profiler times single passes, so it sees the
+// launched ones.
+bool use_loop(const qpat_ctx* c, int batch) {
+  if (!c->loop_on || c->prof_phase >= 0) return false;
+  return loop_waves(c->loop, batch) <= 1 || (c->loop.own_kernel && !(c->pf.fast_rows && c->pf.fast_cols));
+}
+
+// seq_forward and seq_adjoint on the whole-loop kernel: one launch, or one per
+// checkpoint interval when checkpoints are stored.
+long long seq_loop_forward(qpat_ctx* c, int batch, cudaStream_t s, int K, bool store, int resume_m) {
+  const int nt = c->nt, ll = c->cfg.lossless != 0, P = ll ? 4 : 6;
+  int g = ll ? -1 : -2;
+  long long cnt = 0;
+  if (resume_m >= 0) {
+    launch_ckpt_copy<float>(c->pf, batch, resume_m, 0, s);
+    g = (resume_m + 1) * K * P;
+  }
+  const int end = (nt - 1) * P + (ll ? 0 : 1);
+  int load = resume_m >= 0;
+  if (store && K > 0)
+    for (int m = 0; m < (nt - 1) / K; ++m) {
+      const int g1 = (m + 1) * K * P;
+      launch_loop(c->pf, c->loop, 0, ll, batch, nt, g, g1, load, 1, 0, s);
+      launch_ckpt_copy<float>(c->pf, batch, m, 1, s);
+      g = g1;
+      load = 1;
+      ++cnt;
+    }
+  launch_loop(c->pf, c->loop, 0, ll, batch, nt, g, end, load, 0, 1, s);
+  return cnt + 1;
+}
+
+long long seq_loop_adjoint(qpat_ctx* c, int batch, cudaStream_t s) {
+  const int ll = c->cfg.lossless != 0;
+  launch_loop(c->pf, c->loop, 1, ll, batch, c->nt, 0, c->nt * (ll ? 4 : 6) - 3, 0, 0, 0, s);
+  return 1;
+}
+
 // H_a: launch sequence of the forward loop n = -1 .. Nt - 2 (Section 3.2.3),
 // enqueued on stream s; the caller's buffers are read through a.io.
 // Checkpointing (K > 0): after loop iteration n with (n + 1) % K == 0 the
@@ -572,6 +627,7 @@ void pass(qpat_ctx* c, const PropArgs<T>& a, int phase, int batch, bool is_row, 
 // samples (resume_m + 1) K .. Nt - 1 only.
 template <typename T>
 long long seq_forward(qpat_ctx* c, int batch, cudaStream_t s, int K = 0, bool store = false, int resume_m = -1) {
+  if (std::is_same<T, float>::value && use_loop(c, batch)) return seq_loop_forward(c, batch, s, K, store, resume_m);
   PropArgs<T> a = args<T>(c);
   long long cnt = 0;
   const int nt = c->nt;
@@ -634,6 +690,7 @@ long long seq_forward(qpat_ctx* c, int batch, cudaStream_t s, int K = 0, bool st
 // H_a^*: transposed steps in reverse, n = Nt - 2 .. -1 (Section 3.2.4).
 template <typename T>
 long long seq_adjoint(qpat_ctx* c, int batch, cudaStream_t s) {
+  if (std::is_same<T, float>::value && use_loop(c, batch)) return seq_loop_adjoint(c, batch, s);
   PropArgs<T> a = args<T>(c);
   long long cnt = 0;
   zero_state<T>(c, batch, s);
@@ -1640,9 +1697,13 @@ qpat_status qpat_autotune(qpat_ctx* c, int batch, int steps, int* choice) {
   float best = 1e30f;
   int best_choice = 0;
   c->nt = nt_try;
-  for (int cand = 0; cand < 4; ++cand) {
+  bool best_loop = false;
+  for (int cand = 0; cand < 5; ++cand) {
+    const bool loop = cand == 4;                // the whole-loop kernel, last
     const int fr = cand & 1, fc = (cand >> 1) & 1;
-    if ((fr && !rows_ok) || (fc && !cols_ok)) continue;
+    if (!loop && ((fr && !rows_ok) || (fc && !cols_ok))) continue;
+    c->loop_on = loop && c->loop.ok;
+    if (loop && !use_loop(c, batch)) continue;
     c->pf.fast_rows = c->pd.fast_rows = fr;
     c->pf.fast_cols = c->pd.fast_cols = fc;
     float total = 0.f;
@@ -1660,11 +1721,13 @@ qpat_status qpat_autotune(qpat_ctx* c, int batch, int steps, int* choice) {
       cudaEventElapsedTime(&ms, e0, e1);
       if (rep == 1) total = ms;
     }
-    if (total < best) { best = total; best_choice = cand; }
+    if (total < best) { best = total; best_choice = loop ? 3 : cand; best_loop = loop; }
   }
   c->nt = nt_saved;
-  c->pf.fast_rows = c->pd.fast_rows = best_choice & 1;
-  c->pf.fast_cols = c->pd.fast_cols = (best_choice >> 1) & 1;
+  c->loop_on = best_loop;
+  if (best_loop) best_choice = 3;
+  c->pf.fast_rows = c->pd.fast_rows = rows_ok && (best_choice & 1);
+  c->pf.fast_cols = c->pd.fast_cols = cols_ok && ((best_choice >> 1) & 1);
   for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second.first);
   c->graphs.clear();
   cudaEventDestroy(e0);

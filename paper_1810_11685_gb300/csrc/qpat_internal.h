@@ -92,6 +92,7 @@ struct PropArgs {
   const T* sw;
   const int* rowptr;      // [ny + 1] range of grid points per row
   const int* pcol;        // [npts] column of each grid point
+  const int* prow;        // [npts] row of each grid point
   const int* pent;        // [npts + 1] range of (sensor, weight) entries per point
   const int* esens;
   const T* ew;
