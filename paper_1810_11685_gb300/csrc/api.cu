@@ -401,6 +401,14 @@ qpat_status build_context(qpat_ctx* c, const qpat_medium* med, const double* sen
   if (row_smem_bytes<T>(c->nx) > 227 * 1024 || col_smem_bytes<T>(c->ny, a.cb) > 227 * 1024)
     return fail(c, QPAT_EINVAL, "grid too large for the shared-memory FFT passes");
   a.dt = (T)c->dt;
+  a.su = a.sy = a.st = a.sa = (T)1;
+  if (!c->cfg.lossless) {
+    const double t = std::min(1e3, std::max(1e-3, fabs(tan(M_PI * c->cfg.y / 2.0))));
+    auto pow2 = [](double v) { return (T)exp2(round(log2(v))); };
+    a.su = pow2(8.0 * c->dt);
+    a.sy = a.st = pow2(c->c_ref * t);
+    a.sa = pow2(c->dt);
+  }
   const long long G = c->G, N = c->N;
   const int B = c->maxb;
   TableOut<T> o{};
@@ -447,6 +455,19 @@ qpat_status build_context(qpat_ctx* c, const qpat_medium* med, const double* sen
   a.fast_rows = !c->cfg.generic_fft && fast_rows_supported(c->nx, (int)sizeof(T));
   a.fast_cols = !c->cfg.generic_fft && fast_cols_supported(c->ny, (int)sizeof(T));
 
+  if (a.fast_rows) {
+    int q[3];
+    fast_plan(c->nx, q);
+    // (the reversed plan of two stages is its two radices swapped)
+    const int ri[3] = {q[2] > 1 ? q[2] : q[1], q[2] > 1 ? q[1] : q[0], q[2] > 1 ? q[0] : 1};
+    const int nf = stage_twiddle_count(q[0], q[1], q[2]), ni = stage_twiddle_count(ri[0], ri[1], ri[2]);
+    C* tw;
+    QCK(dalloc(c, &tw, (size_t)(nf + ni) * sizeof(C)));
+    QCK(stage_twiddles<T>(q, tw, c->stream));
+    QCK(stage_twiddles<T>(ri, tw + nf, c->stream));
+    a.twxf = tw;
+    a.twxi = tw + nf;
+  }
   // sensors: bilinear weights on the node grid (gather form) and the
   // transposed scatter as a per-row, per-point gather (deterministic)
   std::vector<int> sidx(4 * (size_t)c->ns);
@@ -537,7 +558,7 @@ qpat_status build_context(qpat_ctx* c, const qpat_medium* med, const double* sen
   prop_init_attributes<T>(c->nx, c->ny, a.fast_rows, a.fast_cols);
   if constexpr (std::is_same<T, float>::value) {
     // (cfg.generic_fft asks for the generic passes)
-    if (!c->cfg.generic_fft) loop_plan(a, c->cfg.lossless, c->maxb, c->c_ref, c->dt, c->cfg.y, &c->loop);
+    if (!c->cfg.generic_fft) loop_plan(a, c->cfg.lossless, c->maxb, &c->loop);
     c->loop_on = c->loop.ok;
   }
   return QPAT_OK;

@@ -1,18 +1,17 @@
 // Length-specialised propagation passes on compile-time Stockham FFTs.
 //
 // Row pass (one thread group per pair of grid rows j0, j0 + 1):
-//   load the incoming half spectra straight into registers, Hermitian-extend
-//   them and pack the two rows into one complex sequence -> inverse x-FFT via
-//   conj(FFT(conj .)) with the radices of the forward plan reversed -> each
-//   thread ends holding grid points j + r L/Q1 of both rows -> pointwise
-//   update (row_point) in registers -> forward x-FFT, whose first stage reads
-//   exactly those registers -> split into two half spectra through shared
-//   memory -> store.
+//   load the incoming spectra of both rows (two fields of a row form one complex
+//   sequence; of one field, the two rows do) -> inverse x-FFT via conj(FFT(conj .))
+//   with the radices of the forward plan reversed -> each thread ends holding grid
+//   points j + r L/Q1 of both rows -> pointwise update (row_point) in registers ->
+//   forward x-FFT, whose first stage reads exactly those registers -> store (one
+//   field: split into two half spectra through shared memory first).
 // Column pass (one thread group per half-spectrum column, CBW adjacent
 //   columns per CTA, column index fastest so that global accesses of a warp
 //   are contiguous):
-//   load rows j + r L/Q1 of the column -> forward y-FFT -> spectral symbol
-//   (col_point) on the registers -> inverse y-FFT (reversed radices), which
+//   load rows j + r L/Q1 of the column -> forward y-FFT -> spectral products
+//   (packed_col) on the registers -> inverse y-FFT (reversed radices), which
 //   ends in the load layout -> store.
 #pragma once
 #include "fft_reg.cuh"
@@ -88,19 +87,30 @@ row_fast(const PropArgs<T> a) {
     for (int rr = 0; rr < 2; ++rr)
       st[rr][r] = (j < L / Q1 && valid) ? row_load<T>(a, ph, b, j + r * (L / Q1), j0 + rr) : RowIn<T>{};
 
-  // 1. inverse x-transform of the incoming half spectra (reversed plan)
+  // PML factors of this thread's points
+  T px[Q1], py[2];
+#pragma unroll
+  for (int r = 0; r < Q1; ++r) px[r] = j < L / Q1 ? row_pml_x(a, ph, j + r * (L / Q1)) : (T)0;
+  py[0] = row_pml_y(a, ph, j0);
+  py[1] = row_pml_y(a, ph, j0 + 1);
+
+  // 1. inverse x-transform of the incoming spectra (reversed plan)
   C y[KIN][Q1];
   if (!skip_in) {
     C v[KIN][P1];
     if (j < L / P1) {
 #pragma unroll
       for (int s = 0; s < KIN; ++s) {
-        const C* r0 = spec + s * slot + (long long)j0 * a.pitch;
-        const C* r1 = r0 + a.pitch;
+        const C* r0 = spec + (long long)(j0 + (KIN == 2 ? s : 0)) * a.pitch;
+        const C* r1 = r0 + (KIN == 2 ? slot : a.pitch);
 #pragma unroll
         for (int r = 0; r < P1; ++r) {
           const int n = j + r * (L / P1);
-          C P, Q;
+          if (KIN == 2) {                                // r0, r1: the two slots of row j0 + s
+            v[s][r] = packed_in(r0, r1, n, L);
+            continue;
+          }
+          C P, Q;                                        // r0, r1: rows j0, j0 + 1
           if (2 * n <= L) {
             P = r0[n];
             Q = r1[n];
@@ -130,7 +140,8 @@ row_fast(const PropArgs<T> a) {
   }
 
   // 2. pointwise update on grid points i = j + r L/Q1 of both rows;
-  //    y = FFT(conj Z) = conj(z): row j0 is Re, row j0+1 is -Im
+  //    y = FFT(conj Z) = conj(z): of row j0 + rr, field 0 is Re and field 1 -Im;
+  //    of one field, row j0 is Re and row j0 + 1 -Im
   C o[KOUT][Q1];
   bool bad = false;
 #pragma unroll
@@ -140,14 +151,18 @@ row_fast(const PropArgs<T> a) {
       const int i = j + r * (L / Q1);
 #pragma unroll
       for (int rr = 0; rr < 2; ++rr) {
-        const T in0 = rr ? -y[0][r].y : y[0][r].x;
-        const T in1 = (KIN > 1) ? (rr ? -y[KIN - 1][r].y : y[KIN - 1][r].x) : (T)0;
+        const T in0 = KIN == 2 ? y[KIN == 2 ? rr : 0][r].x : rr ? -y[0][r].y : y[0][r].x;
+        const T in1 = KIN == 2 ? mul_rn(-y[KIN == 2 ? rr : 0][r].y, in1_scale(a, ph)) : (T)0;
         const T scv = (KIN == 1) ? sc[rr * L + i] : (T)0;
-        row_point<T>(a, ph, b, i, j0 + rr, in0, in1, scv, st[rr][r], u0[rr], u1[rr], bad);
+        row_point<T>(a, ph, b, i, j0 + rr, in0, in1, scv, st[rr][r], px[r], py[rr], u0[rr], u1[rr], bad);
       }
     }
-    o[0][r] = cmake<C>(u0[0], u0[1]);
-    if (KOUT > 1) o[KOUT - 1][r] = cmake<C>(u1[0], u1[1]);
+    if (KOUT == 2) {
+      o[0][r] = cmake<C>(u0[0], mul_rn(u1[0], out1_scale(a, ph)));
+      o[KOUT - 1][r] = cmake<C>(u0[1], mul_rn(u1[1], out1_scale(a, ph)));
+    } else {
+      o[0][r] = cmake<C>(u0[0], u0[1]);
+    }
   }
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(a.err, 1);
   if (a.flags & kSkipOutput) return;
@@ -157,6 +172,17 @@ row_fast(const PropArgs<T> a) {
   fft_stockham<L, G::Q1, G::Q2, G::Q3, KOUT>(o, X, bufA, bufB, SL, j, tws);
   // thread j < L/QL holds Z[j + r L/QL]; split Z into the two rows' half
   // spectra A(k) = (Z(k) + conj Z(-k))/2, B(k) = -i (Z(k) - conj Z(-k))/2
+  if constexpr (KOUT == 2) {                       // straight from registers
+    if (j < L / QL && valid) {
+#pragma unroll
+      for (int s = 0; s < KOUT; ++s) {
+        C* w0 = spec + (long long)(j0 + s) * a.pitch;
+#pragma unroll
+        for (int r = 0; r < QL; ++r) packed_out(w0, w0 + slot, j + r * (L / QL), L, X[s][r]);
+      }
+    }
+    return;
+  }
   if (j < L / QL) {
 #pragma unroll
     for (int s = 0; s < KOUT; ++s)
@@ -193,9 +219,10 @@ __host__ __device__ constexpr int row_field(int ph, int v) {
   switch (ph) {
     case F_R1: { const int f[5] = {RFRX, RFRY, RFCC, RFETA, RFTAU}; return f[v]; }
     case F_R2: case A_R5: { const int f[5] = {RFVX, RFVY, RFDX, RFDY, -1}; return f[v]; }
-    case F_R3: case F_R3L: case A_R1L: { const int f[5] = {RFRX, RFRY, RFRHO, RFCC, -1}; return f[v]; }
+    case F_R3: { const int f[5] = {RFRX, RFRY, RFRHO, -1, -1}; return f[v]; }
+    case F_R3L: case A_R1L: { const int f[5] = {RFRX, RFRY, RFRHO, RFCC, -1}; return f[v]; }
     case A_R1: { const int f[5] = {-1, -1, RFCC, RFETA, RFTAU}; return f[v]; }
-    case A_R3: { const int f[5] = {RFRX, RFRY, RFRHO, RFCC, RFPB}; return f[v]; }
+    case A_R3: { const int f[5] = {RFRX, RFRY, RFRHO, -1, RFPB}; return f[v]; }
     default: return -1;
   }
 }
@@ -226,12 +253,10 @@ __device__ __forceinline__ const T* row_field_ptr(const PropArgs<T>& a, int f, i
   }
 }
 
-// c^2 is read by F_R3 and A_R3 only at the source steps.
-__device__ __forceinline__ bool row_field_needed(int ph, int f, int flags) {
-  if (f != RFCC) return true;
-  if (ph == F_R3) return (flags & kSource) != 0;
-  if (ph == A_R3) return (flags & (kAccWrite | kAccAdd)) != 0;
-  return true;
+// F_R3 and A_R3 read c^2 at the source steps only: from global memory there, so
+// that the others need no room for it (576^2 batch 12: 45.1 -> 44.7 ms).
+__device__ __forceinline__ bool row_cc_from_global(int ph, int flags) {
+  return (ph == F_R3 && (flags & kSource)) || (ph == A_R3 && (flags & (kAccWrite | kAccAdd)));
 }
 
 #ifndef QPAT_ROW_STAGED
@@ -259,27 +284,20 @@ __host__ __device__ constexpr int rp_st() { return QPAT_ROWST_RP; }
 #endif
 constexpr bool kRowStOneBuf = QPAT_ROWST_ONEBUF != 0;
 
-// Complex values before the staging area (twiddles and Stockham buffers),
-// rounded up to a 16-byte boundary.
-// Stage twiddles W_L^m of the staged row pass: a per-CTA shared copy (0),
-// which the bulk-copy form fetches with one more copy, or read straight from
-// global memory through L1 (1).  Measured on GB300 at 576^2 batch 12, N_t
-// 600, with bulk copies: 2.352e10 against 2.322e10 cell-steps/s from L1
-// (with per-thread copies the L1 reads were the faster form).
-#ifndef QPAT_ROWST_TWG
-#define QPAT_ROWST_TWG 0
-#endif
-constexpr bool kRowStTwGlobal = QPAT_ROWST_TWG != 0;
-constexpr int kRowStTwSmem(int L) { return kRowStTwGlobal ? 0 : L; }
-
+// Complex values before the staging area (the Stockham buffers), rounded up to a
+// 16-byte boundary.  The stage twiddles are read through L1 from tables in the
+// order of the reads (PropArgs twxf, twxi): from a shared copy of W_L^m the
+// strided reads of the later stages took more shared-memory wavefronts than the
+// data (576^2 batch 12, 150 steps, forward + adjoint: 49.5 -> 45.1 ms, with the
+// PML factors loaded before the transforms).
 template <int L, int NSX, int RP = rp_st<L>()>
 __host__ __device__ constexpr int row_st_offset() {
-  return (kRowStTwSmem(L) + RP * (kRowStOneBuf ? 1 : 2) * NSX * SGeom<L>::SL + 1) & ~1;
+  return (RP * (kRowStOneBuf ? 1 : 2) * NSX * SGeom<L>::SL + 1) & ~1;
 }
 
 // At least six resident CTAs per SM (registers capped to fit; measured at
-// 576^2 batch 12, Nt 600: 2.145e10 with no bound, 2.186e10 with 6, 2.148e10
-// with 7, 2.163e10 with 8 cell-steps/s).
+// 576^2 batch 12 / 1080^2 batch 4: 44.7 / 39.3 ms with 6, 44.4 / 40.6 with 7,
+// 44.7 / 41.9 with 8).
 #ifndef QPAT_ROWST_MINB
 #define QPAT_ROWST_MINB 6
 #endif
@@ -303,9 +321,7 @@ __device__ __forceinline__ void row_st_body(const PropArgs<T> a, const int b, co
   const int m = threadIdx.x / TPT;
   const int j = threadIdx.x - m * TPT;
   C* const sbase = reinterpret_cast<C*>(smem_raw);
-  C* tws = sbase;                                                // W_L^m table
-  const C* tw = kRowStTwGlobal ? a.twx : tws;
-  C* bufA = sbase + kRowStTwSmem(L) + m * NB * NSX * SL;
+  C* bufA = sbase + m * NB * NSX * SL;
   C* bufB = kRowStOneBuf ? bufA : bufA + NSX * SL;
   constexpr int OFF = row_st_offset<L, NSX, RP>();
   T* stage = reinterpret_cast<T*>(sbase + OFF) + m * NF * 2 * L;
@@ -325,7 +341,7 @@ __device__ __forceinline__ void row_st_body(const PropArgs<T> a, const int b, co
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       const int f = row_field(ph, v);
-      if (f < 0 || !row_field_needed(ph, f, a.flags)) continue;
+      if (f < 0) continue;
       const int sl = row_stage_slot(ph, v);
 #pragma unroll
       for (int rr = 0; rr < 2; ++rr) {
@@ -335,22 +351,31 @@ __device__ __forceinline__ void row_st_body(const PropArgs<T> a, const int b, co
       }
     }
   }
-  if constexpr (!kRowStTwGlobal)
-    for (int t = threadIdx.x; t < L; t += RP * TPT) tws[t] = a.twx[t];
 
-  // 1. inverse x-transform of the incoming half spectra (reversed plan)
+  // PML factors of this thread's points
+  T px[Q1], py[2];
+#pragma unroll
+  for (int r = 0; r < Q1; ++r) px[r] = j < L / Q1 ? row_pml_x(a, ph, j + r * (L / Q1)) : (T)0;
+  py[0] = row_pml_y(a, ph, j0);
+  py[1] = row_pml_y(a, ph, j0 + 1);
+
+  // 1. inverse x-transform of the incoming spectra (reversed plan)
   C y[KIN][Q1];
   if (!skip_in) {
     C v[KIN][P1];
     if (j < L / P1) {
 #pragma unroll
       for (int s = 0; s < KIN; ++s) {
-        const C* r0 = spec + s * slot + (long long)j0 * a.pitch;
-        const C* r1 = r0 + a.pitch;
+        const C* r0 = spec + (long long)(j0 + (KIN == 2 ? s : 0)) * a.pitch;
+        const C* r1 = r0 + (KIN == 2 ? slot : a.pitch);
 #pragma unroll
         for (int r = 0; r < P1; ++r) {
           const int n = j + r * (L / P1);
-          C P, Q;
+          if (KIN == 2) {                                // r0, r1: the two slots of row j0 + s
+            v[s][r] = packed_in(r0, r1, n, L);
+            continue;
+          }
+          C P, Q;                                        // r0, r1: rows j0, j0 + 1
           if (2 * n <= L) {
             P = r0[n];
             Q = r1[n];
@@ -363,7 +388,7 @@ __device__ __forceinline__ void row_st_body(const PropArgs<T> a, const int b, co
         }
       }
     }
-    fft_stockham<L, G::P1, G::P2, G::P3, KIN, kRowStOneBuf>(v, y, bufA, bufB, SL, j, tw);
+    fft_stockham<L, G::P1, G::P2, G::P3, KIN, kRowStOneBuf, true, true>(v, y, bufA, bufB, SL, j, a.twxi);
   } else {
 #pragma unroll
     for (int s = 0; s < KIN; ++s)
@@ -381,7 +406,8 @@ __device__ __forceinline__ void row_st_body(const PropArgs<T> a, const int b, co
   __syncthreads();
 
   // 2. pointwise update on grid points i = j + r L/Q1 of both rows;
-  //    y = FFT(conj Z) = conj(z): row j0 is Re, row j0+1 is -Im
+  //    y = FFT(conj Z) = conj(z): of row j0 + rr, field 0 is Re and field 1 -Im;
+  //    of one field, row j0 is Re and row j0 + 1 -Im
   C o[KOUT][Q1];
   bool bad = false;
 #pragma unroll
@@ -395,22 +421,38 @@ __device__ __forceinline__ void row_st_body(const PropArgs<T> a, const int b, co
 #pragma unroll
         for (int v = 0; v < 5; ++v)
           sv[v] = row_field(ph, v) >= 0 ? stage[(row_stage_slot(ph, v) * 2 + rr) * L + i] : (T)0;
+        if (row_cc_from_global(ph, a.flags)) sv[3] = a.Cc[(long long)(j0 + rr) * a.nx + i];
         const RowIn<T> st{sv[0], sv[1], sv[2], sv[3], sv[4]};
-        const T in0 = rr ? -y[0][r].y : y[0][r].x;
-        const T in1 = (KIN > 1) ? (rr ? -y[KIN - 1][r].y : y[KIN - 1][r].x) : (T)0;
+        const T in0 = KIN == 2 ? y[KIN == 2 ? rr : 0][r].x : rr ? -y[0][r].y : y[0][r].x;
+        const T in1 = KIN == 2 ? mul_rn(-y[KIN == 2 ? rr : 0][r].y, in1_scale(a, ph)) : (T)0;
         const T scv = (KIN == 1) ? sc[rr * L + i] : (T)0;
-        row_point<T>(a, ph, b, i, j0 + rr, in0, in1, scv, st, u0[rr], u1[rr], bad);
+        row_point<T>(a, ph, b, i, j0 + rr, in0, in1, scv, st, px[r], py[rr], u0[rr], u1[rr], bad);
       }
     }
-    o[0][r] = cmake<C>(u0[0], u0[1]);
-    if (KOUT > 1) o[KOUT - 1][r] = cmake<C>(u1[0], u1[1]);
+    if (KOUT == 2) {
+      o[0][r] = cmake<C>(u0[0], mul_rn(u1[0], out1_scale(a, ph)));
+      o[KOUT - 1][r] = cmake<C>(u0[1], mul_rn(u1[1], out1_scale(a, ph)));
+    } else {
+      o[0][r] = cmake<C>(u0[0], u0[1]);
+    }
   }
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(a.err, 1);
   if (a.flags & kSkipOutput) return;
 
   // 3. forward x-transform of the packed outgoing rows, split, store
   C X[KOUT][QL];
-  fft_stockham<L, G::Q1, G::Q2, G::Q3, KOUT, kRowStOneBuf>(o, X, bufA, bufB, SL, j, tw);
+  fft_stockham<L, G::Q1, G::Q2, G::Q3, KOUT, kRowStOneBuf, true, true>(o, X, bufA, bufB, SL, j, a.twxf);
+  if constexpr (KOUT == 2) {                       // straight from registers
+    if (j < L / QL && valid) {
+#pragma unroll
+      for (int s = 0; s < KOUT; ++s) {
+        C* w0 = spec + (long long)(j0 + s) * a.pitch;
+#pragma unroll
+        for (int r = 0; r < QL; ++r) packed_out(w0, w0 + slot, j + r * (L / QL), L, X[s][r]);
+      }
+    }
+    return;
+  }
   if (j < L / QL) {
 #pragma unroll
     for (int s = 0; s < KOUT; ++s)
@@ -488,9 +530,7 @@ row_fast_st(const PropArgs<T> a) {
   const int m = threadIdx.x / TPT;
   const int j = threadIdx.x - m * TPT;
   C* const sbase = reinterpret_cast<C*>(smem_raw);
-  C* tws = sbase;                                                // W_L^m table
-  const C* tw = kRowStTwGlobal ? a.twx : tws;
-  C* bufA = sbase + kRowStTwSmem(L) + m * NB * NSX * SL;
+  C* bufA = sbase + m * NB * NSX * SL;
   C* bufB = kRowStOneBuf ? bufA : bufA + NSX * SL;
   constexpr int OFF = row_st_offset<L, NSX>();
   T* stage = reinterpret_cast<T*>(sbase + OFF) + m * NF * 2 * L;
@@ -521,10 +561,7 @@ row_fast_st(const PropArgs<T> a) {
   __syncthreads();
   if (threadIdx.x == 0) {
     const bool load_in = valid && !skip_in;
-    // (with the twiddles in shared memory, they come by one more copy)
-    mbar_arrive_expect_tx(bar, (load_in ? 2u * KIN * kSpecRow * (unsigned)sizeof(C) : 0u) +
-                                   (kRowStTwGlobal ? 0u : L * (unsigned)sizeof(C)));
-    if constexpr (!kRowStTwGlobal) bulk_g2s(tws, a.twx, L * (unsigned)sizeof(C), bar);
+    mbar_arrive_expect_tx(bar, load_in ? 2u * KIN * kSpecRow * (unsigned)sizeof(C) : 0u);
     if (load_in)
       for (int s = 0; s < KIN; ++s)
         for (int rr = 0; rr < 2; ++rr)
@@ -535,7 +572,7 @@ row_fast_st(const PropArgs<T> a) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         const int f = row_field(ph, v);
-        if (f >= 0 && row_field_needed(ph, f, a.flags)) bytes += 2u * L * (unsigned)sizeof(T);
+        if (f >= 0) bytes += 2u * L * (unsigned)sizeof(T);
       }
     }
     mbar_arrive_expect_tx(bar + 1, bytes);
@@ -543,7 +580,7 @@ row_fast_st(const PropArgs<T> a) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         const int f = row_field(ph, v);
-        if (f < 0 || !row_field_needed(ph, f, a.flags)) continue;
+        if (f < 0) continue;
         const int sl = row_stage_slot(ph, v);
         for (int rr = 0; rr < 2; ++rr)
           bulk_g2s(stage + (sl * 2 + rr) * L, row_field_ptr<T>(a, f, b, j0 + rr), L * (unsigned)sizeof(T),
@@ -560,7 +597,7 @@ row_fast_st(const PropArgs<T> a) {
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       const int f = row_field(ph, v);
-      if (f < 0 || !row_field_needed(ph, f, a.flags)) continue;
+      if (f < 0) continue;
       const int sl = row_stage_slot(ph, v);
 #pragma unroll
       for (int rr = 0; rr < 2; ++rr) {
@@ -571,14 +608,18 @@ row_fast_st(const PropArgs<T> a) {
     }
   }
 #endif
+  // PML factors of this thread's points
+  T px[Q1], py[2];
+#pragma unroll
+  for (int r = 0; r < Q1; ++r) px[r] = j < L / Q1 ? row_pml_x(a, ph, j + r * (L / Q1)) : (T)0;
+  py[0] = row_pml_y(a, ph, j0);
+  py[1] = row_pml_y(a, ph, j0 + 1);
+
 #if QPAT_ROWST_BULK
-  row_bulk_wait(bar, a.err);                                     // spectra (and twiddles) in shared memory
-#else
-  if constexpr (!kRowStTwGlobal)
-    for (int t = threadIdx.x; t < L; t += blockDim.x) tws[t] = a.twx[t];
+  row_bulk_wait(bar, a.err);                                     // spectra in shared memory
 #endif
 
-  // 1. inverse x-transform of the incoming half spectra (reversed plan)
+  // 1. inverse x-transform of the incoming spectra (reversed plan)
   C y[KIN][Q1];
   if (!skip_in) {
     C v[KIN][P1];
@@ -586,16 +627,20 @@ row_fast_st(const PropArgs<T> a) {
 #pragma unroll
       for (int s = 0; s < KIN; ++s) {
 #if QPAT_ROWST_BULK
-        const C* r0 = sp + (s * 2) * kSpecRow;
-        const C* r1 = r0 + kSpecRow;
+        const C* r0 = sp + (KIN == 2 ? s : 0) * kSpecRow;        // staged as slot 0 rows, slot 1 rows
+        const C* r1 = r0 + (KIN == 2 ? 2 : 1) * kSpecRow;
 #else
-        const C* r0 = spec + s * slot + (long long)j0 * a.pitch;
-        const C* r1 = r0 + a.pitch;
+        const C* r0 = spec + (long long)(j0 + (KIN == 2 ? s : 0)) * a.pitch;
+        const C* r1 = r0 + (KIN == 2 ? slot : a.pitch);
 #endif
 #pragma unroll
         for (int r = 0; r < P1; ++r) {
           const int n = j + r * (L / P1);
-          C P, Q;
+          if (KIN == 2) {                                // r0, r1: the two slots of row j0 + s
+            v[s][r] = packed_in(r0, r1, n, L);
+            continue;
+          }
+          C P, Q;                                        // r0, r1: rows j0, j0 + 1
           if (2 * n <= L) {
             P = r0[n];
             Q = r1[n];
@@ -611,7 +656,7 @@ row_fast_st(const PropArgs<T> a) {
 #if QPAT_ROWST_BULK
     __syncthreads();                                              // staged spectra read before the first stage writes
 #endif
-    fft_stockham<L, G::P1, G::P2, G::P3, KIN, kRowStOneBuf>(v, y, bufA, bufB, SL, j, tw);
+    fft_stockham<L, G::P1, G::P2, G::P3, KIN, kRowStOneBuf, true, true>(v, y, bufA, bufB, SL, j, a.twxi);
   } else {
 #pragma unroll
     for (int s = 0; s < KIN; ++s)
@@ -633,7 +678,8 @@ row_fast_st(const PropArgs<T> a) {
   __syncthreads();
 
   // 2. pointwise update on grid points i = j + r L/Q1 of both rows;
-  //    y = FFT(conj Z) = conj(z): row j0 is Re, row j0+1 is -Im
+  //    y = FFT(conj Z) = conj(z): of row j0 + rr, field 0 is Re and field 1 -Im;
+  //    of one field, row j0 is Re and row j0 + 1 -Im
   C o[KOUT][Q1];
   bool bad = false;
 #pragma unroll
@@ -647,22 +693,38 @@ row_fast_st(const PropArgs<T> a) {
 #pragma unroll
         for (int v = 0; v < 5; ++v)
           sv[v] = row_field(ph, v) >= 0 ? stage[(row_stage_slot(ph, v) * 2 + rr) * L + i] : (T)0;
+        if (row_cc_from_global(ph, a.flags)) sv[3] = a.Cc[(long long)(j0 + rr) * a.nx + i];
         const RowIn<T> st{sv[0], sv[1], sv[2], sv[3], sv[4]};
-        const T in0 = rr ? -y[0][r].y : y[0][r].x;
-        const T in1 = (KIN > 1) ? (rr ? -y[KIN - 1][r].y : y[KIN - 1][r].x) : (T)0;
+        const T in0 = KIN == 2 ? y[KIN == 2 ? rr : 0][r].x : rr ? -y[0][r].y : y[0][r].x;
+        const T in1 = KIN == 2 ? mul_rn(-y[KIN == 2 ? rr : 0][r].y, in1_scale(a, ph)) : (T)0;
         const T scv = (KIN == 1) ? sc[rr * L + i] : (T)0;
-        row_point<T>(a, ph, b, i, j0 + rr, in0, in1, scv, st, u0[rr], u1[rr], bad);
+        row_point<T>(a, ph, b, i, j0 + rr, in0, in1, scv, st, px[r], py[rr], u0[rr], u1[rr], bad);
       }
     }
-    o[0][r] = cmake<C>(u0[0], u0[1]);
-    if (KOUT > 1) o[KOUT - 1][r] = cmake<C>(u1[0], u1[1]);
+    if (KOUT == 2) {
+      o[0][r] = cmake<C>(u0[0], mul_rn(u1[0], out1_scale(a, ph)));
+      o[KOUT - 1][r] = cmake<C>(u0[1], mul_rn(u1[1], out1_scale(a, ph)));
+    } else {
+      o[0][r] = cmake<C>(u0[0], u0[1]);
+    }
   }
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(a.err, 1);
   if (a.flags & kSkipOutput) return;
 
   // 3. forward x-transform of the packed outgoing rows, split, store
   C X[KOUT][QL];
-  fft_stockham<L, G::Q1, G::Q2, G::Q3, KOUT, kRowStOneBuf>(o, X, bufA, bufB, SL, j, tw);
+  fft_stockham<L, G::Q1, G::Q2, G::Q3, KOUT, kRowStOneBuf, true, true>(o, X, bufA, bufB, SL, j, a.twxf);
+  if constexpr (KOUT == 2) {                       // straight from registers
+    if (j < L / QL && valid) {
+#pragma unroll
+      for (int s = 0; s < KOUT; ++s) {
+        C* w0 = spec + (long long)(j0 + s) * a.pitch;
+#pragma unroll
+        for (int r = 0; r < QL; ++r) packed_out(w0, w0 + slot, j + r * (L / QL), L, X[s][r]);
+      }
+    }
+    return;
+  }
   if (j < L / QL) {
 #pragma unroll
     for (int s = 0; s < KOUT; ++s)
@@ -726,6 +788,7 @@ __device__ __forceinline__ void col_body(const PropArgs<T> a, const int b, const
   const int kx = blk * CBW + c;
   const bool valid = kx < a.nxh;
   const int kxs = valid ? kx : 0;
+  const bool self = kxs == 0 || 2 * kxs == a.nx;
   C* spec = a.spec + (long long)b * a.sstride;
   const long long slot = (long long)a.ny * a.pitch;
 
@@ -736,15 +799,21 @@ __device__ __forceinline__ void col_body(const PropArgs<T> a, const int b, const
 #pragma unroll
     for (int s = 0; s < KIN; ++s)
 #pragma unroll
-      for (int r = 0; r < Q1; ++r) v[s][r] = spec[s * slot + (long long)(j + r * (L / Q1)) * a.pitch + kxs];
+      for (int r = 0; r < Q1; ++r) {
+        // (kx = 0 and kx = nx/2 are their own mirror images: conj of slot 0)
+        const C z = spec[(self ? 0 : s * slot) + (long long)(j + r * (L / Q1)) * a.pitch + kxs];
+        v[s][r] = s == 1 && self ? cconj(z) : z;
+      }
   }
   // twiddles to shared memory and the symbol operands of this thread's
   // points into registers before the transforms
   for (int t = threadIdx.x; t < L; t += CBW * G::TPT) tws[t] = a.twy[t];
   ColIn<T, C> cst[QL];
+  const T k2s = k2_scale(a, ph);
 #pragma unroll
   for (int r = 0; r < QL; ++r)
-    cst[r] = (j < L / QL && valid) ? col_load<T, C>(a, ph, kx, j + r * (L / QL)) : ColIn<T, C>{};
+    cst[r] = (j < L / QL && valid) ? col_half<T, C>(a, ph, col_load<T, C>(a, ph, kx, j + r * (L / QL)), k2s)
+                                   : ColIn<T, C>{};
   const C sx = col_sx<T, C>(a, ph, kxs);
   C X[KIN][QL];
   fft_stockham<L, G::Q1, G::Q2, G::Q3, KIN, false, kColPairs>(v, X, bufA, bufB, SL, j, tws);
@@ -753,7 +822,7 @@ __device__ __forceinline__ void col_body(const PropArgs<T> a, const int b, const
 #pragma unroll
   for (int r = 0; r < QL; ++r) {
     C o0 = cmake<C>((T)0, (T)0), o1 = o0;
-    if (j < L / QL && valid) col_apply<T, C>(ph, cst[r], sx, X[0][r], X[KIN - 1][r], o0, o1);
+    if (j < L / QL && valid) packed_col<T, C>(ph, cst[r], sx, X[0][r], X[KIN - 1][r], o0, o1);
     o[0][r] = cconj(o0);
     if (KOUT > 1) o[KOUT - 1][r] = cconj(o1);
   }
@@ -770,13 +839,13 @@ __device__ __forceinline__ void col_body(const PropArgs<T> a, const int b, const
 
 // The single-context column pass, with its own copy of the body of col_body
 // for the same reason as row_fast_st.
-template <typename T, int L, int PH>
-__global__ void __launch_bounds__(SGeom<L>::CBW * SGeom<L>::TPT)
+template <typename T, int L, int PH, int CBW>
+__global__ void __launch_bounds__(CBW * SGeom<L>::TPT)
 col_fast(const PropArgs<T> a) {
   constexpr int ph = PH, KIN = col_kin(PH), KOUT = col_kout(PH);
   typedef typename V2<T>::t C;
   typedef SGeom<L> G;
-  constexpr int SL = G::SL, CBW = G::CBW, NSX = (KIN > KOUT ? KIN : KOUT);
+  constexpr int SL = G::SL, NSX = (KIN > KOUT ? KIN : KOUT);
   constexpr int Q1 = G::Q1, QL = G::QL;
   constexpr int CS = col_stride<L, NSX, CBW>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -789,6 +858,7 @@ col_fast(const PropArgs<T> a) {
   const int kx = blockIdx.x * CBW + c;
   const bool valid = kx < a.nxh;
   const int kxs = valid ? kx : 0;
+  const bool self = kxs == 0 || 2 * kxs == a.nx;
   C* spec = a.spec + (long long)b * a.sstride;
   const long long slot = (long long)a.ny * a.pitch;
 
@@ -799,15 +869,21 @@ col_fast(const PropArgs<T> a) {
 #pragma unroll
     for (int s = 0; s < KIN; ++s)
 #pragma unroll
-      for (int r = 0; r < Q1; ++r) v[s][r] = spec[s * slot + (long long)(j + r * (L / Q1)) * a.pitch + kxs];
+      for (int r = 0; r < Q1; ++r) {
+        // (kx = 0 and kx = nx/2 are their own mirror images: conj of slot 0)
+        const C z = spec[(self ? 0 : s * slot) + (long long)(j + r * (L / Q1)) * a.pitch + kxs];
+        v[s][r] = s == 1 && self ? cconj(z) : z;
+      }
   }
   // twiddles to shared memory and the symbol operands of this thread's
   // points into registers before the transforms
   for (int t = threadIdx.x; t < L; t += blockDim.x) tws[t] = a.twy[t];
   ColIn<T, C> cst[QL];
+  const T k2s = k2_scale(a, ph);
 #pragma unroll
   for (int r = 0; r < QL; ++r)
-    cst[r] = (j < L / QL && valid) ? col_load<T, C>(a, ph, kx, j + r * (L / QL)) : ColIn<T, C>{};
+    cst[r] = (j < L / QL && valid) ? col_half<T, C>(a, ph, col_load<T, C>(a, ph, kx, j + r * (L / QL)), k2s)
+                                   : ColIn<T, C>{};
   const C sx = col_sx<T, C>(a, ph, kxs);
   C X[KIN][QL];
   fft_stockham<L, G::Q1, G::Q2, G::Q3, KIN, false, kColPairs>(v, X, bufA, bufB, SL, j, tws);
@@ -816,7 +892,7 @@ col_fast(const PropArgs<T> a) {
 #pragma unroll
   for (int r = 0; r < QL; ++r) {
     C o0 = cmake<C>((T)0, (T)0), o1 = o0;
-    if (j < L / QL && valid) col_apply<T, C>(ph, cst[r], sx, X[0][r], X[KIN - 1][r], o0, o1);
+    if (j < L / QL && valid) packed_col<T, C>(ph, cst[r], sx, X[0][r], X[KIN - 1][r], o0, o1);
     o[0][r] = cconj(o0);
     if (KOUT > 1) o[KOUT - 1][r] = cconj(o1);
   }
@@ -856,10 +932,21 @@ void set_row_fast_attr() {
     cudaFuncSetAttribute(row_fast<T, L, PH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)row_fast_smem<T, L, PH>());
 }
+// Extents whose column pass also has a form of 2 columns per CTA, for launches
+// whose wide CTAs fill at most half of the SMs (576^2, 100 steps, forward +
+// adjoint, wide / narrow: one problem 8.4 / 6.5 ms, two 9.0 / 8.4, three 10.1 /
+// 10.7; 288^2, one problem 5.8 / 5.5 ms, four 6.2 / 6.3).
+template <int L>
+constexpr bool col_narrow() { return L >= 168; }
+
 template <typename T, int L, int PH>
 void set_col_fast_attr() {
   static_assert(col_fast_smem<T, L, PH>() <= 227 * 1024, "column pass shared memory above the 227 KB a CTA may use");
-  cudaFuncSetAttribute(col_fast<T, L, PH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)col_fast_smem<T, L, PH>());
+  cudaFuncSetAttribute(col_fast<T, L, PH, SGeom<L>::CBW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)col_fast_smem<T, L, PH>());
+  if constexpr (col_narrow<L>())
+    cudaFuncSetAttribute(col_fast<T, L, PH, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)col_fast_smem<T, L, PH, 2>());
 }
 
 // Dynamic shared-memory limits of all pass kernels of length L; called at
@@ -889,8 +976,14 @@ void run_row_fast(const PropArgs<T>& a, int batch, cudaStream_t s) {
 template <typename T, int L, int PH>
 void run_col_fast(const PropArgs<T>& a, int batch, cudaStream_t s) {
   typedef SGeom<L> G;
+  if constexpr (col_narrow<L>()) {
+    if ((a.nxh + G::CBW - 1) / G::CBW * batch <= kSMs / 2) {
+      col_fast<T, L, PH, 2><<<dim3((a.nxh + 1) / 2, batch), 2 * G::TPT, col_fast_smem<T, L, PH, 2>(), s>>>(a);
+      return;
+    }
+  }
   dim3 grid((a.nxh + G::CBW - 1) / G::CBW, batch);
-  col_fast<T, L, PH><<<grid, G::CBW * G::TPT, col_fast_smem<T, L, PH>(), s>>>(a);
+  col_fast<T, L, PH, G::CBW><<<grid, G::CBW * G::TPT, col_fast_smem<T, L, PH>(), s>>>(a);
 }
 
 // Entry points of one specialised length L (one translation unit each).

@@ -177,14 +177,17 @@ __device__ __forceinline__ P2 p2_from(float4 f) { return P2{F2(f.x, f.y), F2(f.z
 // Twiddle and DFT of one radix-R butterfly of a stage with stride Ns, for NS
 // sequences at once.  a[s][r] = x_s[j + r L/R] on entry, the butterfly's
 // outputs (for positions (j/Ns) Ns R + (j mod Ns) + r Ns) on exit.
-template <int L, int R, int Ns, int NS, typename C>
+// The stage's twiddles W_L^(k r step) come from the table W_L^m (exponent below
+// L, no reduction needed) or, STW, from a table of the stage's own at
+// (r - 1) Ns + k, which a warp reads in order (stage_twiddles).
+template <int L, int R, int Ns, int NS, bool STW = false, typename C>
 __device__ __forceinline__ void butterfly(C (&a)[NS][R], int j, const C* __restrict__ tw) {
   if constexpr (Ns > 1) {
     constexpr int step = L / (Ns * R);
     const int k = j % Ns;
 #pragma unroll
     for (int r = 1; r < R; ++r) {
-      const C w = tw[k * r * step];          // exponent < L, no reduction needed
+      const C w = tw[STW ? (r - 1) * Ns + k : k * r * step];
 #pragma unroll
       for (int s = 0; s < NS; ++s) a[s][r] = cmul(a[s][r], w);
     }
@@ -199,14 +202,14 @@ __device__ __forceinline__ int stockham_pos(int j, int r) {
 }
 
 // butterfly() for NP sequence pairs.
-template <int L, int R, int Ns, int NP>
+template <int L, int R, int Ns, int NP, bool STW = false>
 __device__ __forceinline__ void butterfly2(P2 (&a)[NP][R], int j, const float2* __restrict__ tw) {
   if constexpr (Ns > 1) {
     constexpr int step = L / (Ns * R);
     const int k = j % Ns;
 #pragma unroll
     for (int r = 1; r < R; ++r) {
-      const float2 w = tw[k * r * step];
+      const float2 w = tw[STW ? (r - 1) * Ns + k : k * r * step];
 #pragma unroll
       for (int q = 0; q < NP; ++q) a[q][r] = cmul(a[q][r], w);
     }
@@ -249,12 +252,13 @@ __device__ __forceinline__ void st_load(const float2* buf, int sl, P2 (&p)[NP][R
 
 // fft_stockham for NS >= 2 FP32 sequences: pairs of sequences run as packed
 // FP32x2 arithmetic, an odd last sequence as complex float2 values.
-template <int L, int Q1, int Q2, int Q3, int NS, bool ONEBUF>
+template <int L, int Q1, int Q2, int Q3, int NS, bool ONEBUF, bool STW>
 __device__ __forceinline__ void fft_stockham_pairs(float2 (&a1)[NS][Q1], float2 (&a3)[NS][(Q3 > 1 ? Q3 : Q2)],
                                                    float2* bufA, float2* bufB, int sl, int j,
                                                    const float2* __restrict__ tw) {
   constexpr int NP = NS / 2, QL = (Q3 > 1 ? Q3 : Q2);
   constexpr bool ODD = NS % 2 == 1;
+  const float2* const tw3 = STW ? tw + Q1 * (Q2 - 1) : tw;   // third stage's twiddles
   P2 p1[NP][Q1];
   float2 o1[1][Q1];
   if (j < L / Q1) {
@@ -276,24 +280,24 @@ __device__ __forceinline__ void fft_stockham_pairs(float2 (&a1)[NS][Q1], float2 
   if constexpr (Q3 == 1) {
     if (j < L / Q2) {
       st_load<NS, Q2, NP>(bufA, sl, p3, o3, j, L / Q2);
-      butterfly2<L, Q2, Q1, NP>(p3, j, tw);
-      if constexpr (ODD) butterfly<L, Q2, Q1, 1>(o3, j, tw);
+      butterfly2<L, Q2, Q1, NP, STW>(p3, j, tw);
+      if constexpr (ODD) butterfly<L, Q2, Q1, 1, STW>(o3, j, tw);
     }
   } else {
     P2 p2[NP][Q2];
     float2 o2[1][Q2];
     if (j < L / Q2) {
       st_load<NS, Q2, NP>(bufA, sl, p2, o2, j, L / Q2);
-      butterfly2<L, Q2, Q1, NP>(p2, j, tw);
-      if constexpr (ODD) butterfly<L, Q2, Q1, 1>(o2, j, tw);
+      butterfly2<L, Q2, Q1, NP, STW>(p2, j, tw);
+      if constexpr (ODD) butterfly<L, Q2, Q1, 1, STW>(o2, j, tw);
     }
     if constexpr (ONEBUF) __syncthreads();
     if (j < L / Q2) st_store<NS, Q2, NP>(bufB, sl, p2, o2, stockham_pos<Q2, Q1>(j, 0), Q1);
     __syncthreads();
     if (j < L / Q3) {
       st_load<NS, Q3, NP>(bufB, sl, p3, o3, j, L / Q3);
-      butterfly2<L, Q3, Q1 * Q2, NP>(p3, j, tw);
-      if constexpr (ODD) butterfly<L, Q3, Q1 * Q2, 1>(o3, j, tw);
+      butterfly2<L, Q3, Q1 * Q2, NP, STW>(p3, j, tw3);
+      if constexpr (ODD) butterfly<L, Q3, Q1 * Q2, 1, STW>(o3, j, tw3);
     }
   }
   if (j < L / QL) {
@@ -321,12 +325,15 @@ __device__ __forceinline__ void fft_stockham_pairs(float2 (&a1)[NS][Q1], float2 
 // ONEBUF: bufB may alias bufA; the middle stage of a three-stage plan then
 // waits for every thread's reads before its writes (one more barrier, half
 // the shared memory).
-template <int L, int Q1, int Q2, int Q3, int NS, bool ONEBUF = false, bool PAIRS = true, typename C>
+// STW: tw holds the second and third stage's twiddles, each in the order its
+// warps read them (stage_twiddles in tables.cu).
+template <int L, int Q1, int Q2, int Q3, int NS, bool ONEBUF = false, bool PAIRS = true, bool STW = false, typename C>
 __device__ __forceinline__ void fft_stockham(C (&a1)[NS][Q1], C (&a3)[NS][(Q3 > 1 ? Q3 : Q2)], C* bufA, C* bufB,
                                              int sl, int j, const C* __restrict__ tw) {
   static_assert(Q1 * Q2 * Q3 == L, "radices must multiply to L");
+  const C* const tw3 = STW ? tw + Q1 * (Q2 - 1) : tw;
   if constexpr (PAIRS && QPAT_FFT_PAIRS && NS >= 2 && std::is_same<C, float2>::value) {
-    fft_stockham_pairs<L, Q1, Q2, Q3, NS, ONEBUF>(a1, a3, bufA, bufB, sl, j, tw);
+    fft_stockham_pairs<L, Q1, Q2, Q3, NS, ONEBUF, STW>(a1, a3, bufA, bufB, sl, j, tw);
     return;
   }
   if (j < L / Q1) {
@@ -343,7 +350,7 @@ __device__ __forceinline__ void fft_stockham(C (&a1)[NS][Q1], C (&a3)[NS][(Q3 > 
       for (int s = 0; s < NS; ++s)
 #pragma unroll
         for (int r = 0; r < Q2; ++r) a3[s][r] = bufA[s * sl + spad(j + r * (L / Q2))];
-      butterfly<L, Q2, Q1, NS>(a3, j, tw);
+      butterfly<L, Q2, Q1, NS, STW>(a3, j, tw);
     }
   } else if constexpr (ONEBUF) {
     C a2[NS][Q2];
@@ -352,7 +359,7 @@ __device__ __forceinline__ void fft_stockham(C (&a1)[NS][Q1], C (&a3)[NS][(Q3 > 
       for (int s = 0; s < NS; ++s)
 #pragma unroll
         for (int r = 0; r < Q2; ++r) a2[s][r] = bufA[s * sl + spad(j + r * (L / Q2))];
-      butterfly<L, Q2, Q1, NS>(a2, j, tw);
+      butterfly<L, Q2, Q1, NS, STW>(a2, j, tw);
     }
     __syncthreads();
     if (j < L / Q2) {
@@ -367,7 +374,7 @@ __device__ __forceinline__ void fft_stockham(C (&a1)[NS][Q1], C (&a3)[NS][(Q3 > 
       for (int s = 0; s < NS; ++s)
 #pragma unroll
         for (int r = 0; r < Q3; ++r) a3[s][r] = bufB[s * sl + spad(j + r * (L / Q3))];
-      butterfly<L, Q3, Q1 * Q2, NS>(a3, j, tw);
+      butterfly<L, Q3, Q1 * Q2, NS, STW>(a3, j, tw3);
     }
   } else {
     if (j < L / Q2) {
@@ -376,7 +383,7 @@ __device__ __forceinline__ void fft_stockham(C (&a1)[NS][Q1], C (&a3)[NS][(Q3 > 
       for (int s = 0; s < NS; ++s)
 #pragma unroll
         for (int r = 0; r < Q2; ++r) a2[s][r] = bufA[s * sl + spad(j + r * (L / Q2))];
-      butterfly<L, Q2, Q1, NS>(a2, j, tw);
+      butterfly<L, Q2, Q1, NS, STW>(a2, j, tw);
 #pragma unroll
       for (int s = 0; s < NS; ++s)
 #pragma unroll
@@ -388,7 +395,7 @@ __device__ __forceinline__ void fft_stockham(C (&a1)[NS][Q1], C (&a3)[NS][(Q3 > 
       for (int s = 0; s < NS; ++s)
 #pragma unroll
         for (int r = 0; r < Q3; ++r) a3[s][r] = bufB[s * sl + spad(j + r * (L / Q3))];
-      butterfly<L, Q3, Q1 * Q2, NS>(a3, j, tw);
+      butterfly<L, Q3, Q1 * Q2, NS, STW>(a3, j, tw3);
     }
   }
   __syncthreads();

@@ -1,6 +1,4 @@
 // Host side of the whole-loop kernel (loop2d.cuh): radices, fit and launch.
-#include <math.h>
-
 #include "loop2d.h"
 
 namespace qpat {
@@ -12,7 +10,6 @@ int line_stride(const LoopAxis& x, const LoopAxis& y) {
 }
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 constexpr int kClusters[3] = {16, 8, 4};
-float pow2_near(double v) { return (float)exp2(round(log2(v))); }
 }  // namespace
 
 size_t loop_smem(const PropArgs<float>& a, const LoopAxis& x, const LoopAxis& y, int nc, int adj, int lossless) {
@@ -43,21 +40,13 @@ int occupancy(int L, int adj, int ll, int nc, size_t smem) {
 }
 }  // namespace
 
-void loop_plan(const PropArgs<float>& a, int lossless, int max_batch, double c_ref, double dt, double y_exp,
-               LoopPlan* p) {
+void loop_plan(const PropArgs<float>& a, int lossless, int max_batch, LoopPlan* p) {
   *p = LoopPlan{};
   p->x = loop_axis(a.nx);
   p->y = loop_axis(a.ny);
   if (!p->x.L || !p->y.L) return;
   const int L = kernel_extent(a);
   p->own_kernel = L != 0;
-  if (!lossless) {
-    double t = fabs(tan(M_PI * y_exp / 2.0));
-    t = t < 1e-3 ? 1e-3 : t > 1e3 ? 1e3 : t;
-    p->su = pow2_near(8.0 * dt);
-    p->sy = p->st = pow2_near(c_ref * t);
-    p->sa = pow2_near(dt);
-  }
   // the adjoint kernel holds more than the forward one: it decides the fit
   // (smaller clusters are only looked at when max_batch may not fit as 16s)
   if (!occupancy(L, 0, lossless, 0, 0)) return;
@@ -108,10 +97,6 @@ cudaError_t launch_loop(const PropArgs<float>& a, const LoopPlan& p, int adj, in
   A.load = load;
   A.save = save;
   A.gather_last = gather_last;
-  A.su = p.su;
-  A.sy = p.sy;
-  A.st = p.st;
-  A.sa = p.sa;
   const size_t smem = loop_smem(a, p.x, p.y, nc, adj, lossless);
   switch (kernel_extent(a)) {
 #define QPAT_LOOP_CASE(L) case L: return loop_launch_len<L>(A, adj, lossless, nc, batch, smem, s);

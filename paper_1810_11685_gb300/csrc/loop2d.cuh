@@ -25,8 +25,8 @@
 // transforms are the columns kx and (conjugated) -kx.  A and B are the two
 // lanes of the packed stream.  A single field (the pressure) is packed as two
 // rows p_j + i p_(j+1), which the column pass separates as it loads.
-// Fields that share a transform are balanced by powers of two (LoopPlan), so
-// that neither's rounding drowns the other.
+// Fields that share a transform are balanced by powers of two (PropArgs su to
+// sa), so that neither's rounding drowns the other.
 //
 // Each transform is a Stockham FFT of three stages, with its length known at
 // compile time for the square grids listed in loop2d.h and compile-time
@@ -322,7 +322,7 @@ __device__ __forceinline__ void loop_row_point(const LoopArgs& A, const LoopShar
     if constexpr (PH == F_R3) {
       o0 = rx + ry;
       const F2 ux = F2(ax * r0), uy = F2(ay * r0);
-      o1 = F2(F2(A.su) * F2(F2(ux * f0) + uy * f1));
+      o1 = F2(F2(A.a.su) * F2(F2(ux * f0) + uy * f1));
     } else {
       const F2 pr = F2(F2(S.Cc[p]) * (rx + ry));
       float* pb = a.pbuf + (long long)b * a.gstride + (long long)j0 * nx + i;
@@ -343,7 +343,7 @@ __device__ __forceinline__ void loop_row_point(const LoopArgs& A, const LoopShar
     if constexpr (PH == A_R1L) rpart = F2(F2(S.Cc[p]) * (f0 + F2(S.sc[p])));
     else {
       rpart = F2(S.pb[p]) - f0;
-      ya = F2(f1 * F2(A.sa));                                    
+      ya = F2(f1 * F2(A.a.sa));                                    
     }
     const F2 ax(S.ax[i]), ay(S.ay[m]), r0(S.rho[p]);
     const F2 rtx = F2(S.rx[p]) + rpart, rty = F2(S.ry[p]) + rpart;
@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(loop_threads(LC), 1) loop2d_kernel(const __gri
     S.shp = shp; S.shm = shm; S.ax = pax; S.asx = pasx; S.ay = pay; S.asy = pasy;
   }
   // state, medium, tables
-  const float tau_scale = LL ? 1.f : ADJ ? A.st : A.sy;          
+  const float tau_scale = LL ? 1.f : ADJ ? A.a.st : A.a.sy;          
   for (int t = tid; t < rows * nx; t += NT) {
     const int m = t / nx, i = t - m * nx;
     const long long g = 2LL * (jp0 + m) * nx + i, gb = (long long)b * a.gstride + g;
@@ -626,7 +626,7 @@ __global__ void __launch_bounds__(loop_threads(LC), 1) loop2d_kernel(const __gri
     }
   }
   // (the balance factors are powers of two: scaling a table by them is exact)
-  const float kp2_scale = LL ? 1.f : ADJ ? 1.f / (A.st * A.sa) : 1.f / (A.su * A.sy);
+  const float kp2_scale = LL ? 1.f : ADJ ? 1.f / (A.a.st * A.a.sa) : 1.f / (A.a.su * A.a.sy);
   for (int t = tid; t < cols * ny; t += NT) {
     const int m = t / ny, ky = t - m * ny;
     const long long o = (long long)ky * a.nxh + kx0 + m;

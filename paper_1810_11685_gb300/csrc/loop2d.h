@@ -54,10 +54,6 @@ struct LoopPlan {
   int ok = 0;              // the grid has a plan and one problem fits a cluster
   int own_kernel = 0;      // square grid of an extent with compile-time kernels
   LoopAxis x{}, y{};
-  // Powers of two that balance two fields sharing a transform: with k c ~ omega
-  // and omega dt < 1, u ~ omega sum rho is sent as su u; Y_abs u ~ c k^(y-1) as
-  // Y_abs u / sy; tau Cp as st tau Cp; Y_abs^T tau Cp as Y_abs^T tau Cp / sa.
-  float su = 1.f, sy = 1.f, st = 1.f, sa = 1.f;
   int max_clusters[3] = {0, 0, 0}; // clusters of 16, 8, 4 CTAs resident at once (0: does not fit)
 };
 
@@ -70,7 +66,6 @@ struct LoopArgs {
   int g0, g1;              // passes [g0, g1) of the loop (loop_pass)
   int load, save;          // restore the state from / leave it in the context's arrays
   int gather_last;         // gather sample nt - 1 at the end (forward)
-  float su, sy, st, sa;    // as in LoopPlan
 };
 
 // Shared-memory layout of one CTA in floats (every block a multiple of 16 bytes).
@@ -103,8 +98,8 @@ __host__ __device__ inline LoopLayout loop_layout(const LoopAxis& x, const LoopA
 
 // Shared memory of one CTA of the loop kernel.
 size_t loop_smem(const PropArgs<float>& a, const LoopAxis& x, const LoopAxis& y, int nc, int adj, int lossless);
-// Plan of a grid (y_exp: absorption exponent); sets the kernels' attributes.
-void loop_plan(const PropArgs<float>& a, int lossless, int max_batch, double c_ref, double dt, double y_exp, LoopPlan* p);
+// Plan of a grid; sets the kernels' attributes.
+void loop_plan(const PropArgs<float>& a, int lossless, int max_batch, LoopPlan* p);
 // Rounds of resident clusters that `batch` problems take.
 int loop_waves(const LoopPlan& p, int batch);
 // Passes [g0, g1) of H_a (adj = 0) or H_a^* (adj = 1) of nt samples for

@@ -98,15 +98,26 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
   return false;
 }
 
+// PML factors of a row pass at column i and row j (staggered for the velocity
+// updates), loaded before the transforms.
+template <typename T>
+__device__ __forceinline__ T row_pml_x(const PropArgs<T>& a, const int ph, const int i) {
+  return (ph == F_R2 || ph == A_R5) ? a.asx[i] : (ph == F_R1 || ph == A_R1) ? (T)0 : a.ax[i];
+}
+template <typename T>
+__device__ __forceinline__ T row_pml_y(const PropArgs<T>& a, const int ph, const int j) {
+  return (ph == F_R2 || ph == A_R5) ? a.asy[j] : (ph == F_R1 || ph == A_R1) ? (T)0 : a.ay[j];
+}
+
 // Pointwise update of one grid point (i, j) of problem b in a row pass.
 // in0/in1: the incoming fields after the inverse transforms (already
 // normalised); scv: M^T w at this point (adjoint sensor source, A_R1*);
-// st: the operands from row_load.  Writes the outgoing fields to out0/out1
+// st: the operands from row_load; px, py: row_pml_x, row_pml_y.  Writes the outgoing fields to out0/out1
 // (to be forward transformed) and the updated state to global memory.
 template <typename T>
 __device__ __forceinline__ void row_point(const PropArgs<T>& a, const int ph, const int b, const int i, const int j,
-                                          const T in0, const T in1, const T scv, const RowIn<T>& st, T& out0,
-                                          T& out1, bool& bad) {
+                                          const T in0, const T in1, const T scv, const RowIn<T>& st, const T px,
+                                          const T py, T& out0, T& out1, bool& bad) {
   const long long g = (long long)j * a.nx + i;
   const long long gb = (long long)b * a.gstride;
   const bool interior = (i >= a.pml) && (i < a.pml + a.n0) && (j >= a.pml) && (j < a.pml + a.n1);
@@ -122,7 +133,7 @@ __device__ __forceinline__ void row_point(const PropArgs<T>& a, const int ph, co
     out0 = p;
   } else if (ph == F_R2) {
     // eq. num-vel: v_i <- A_i (A_i v_i - dt/rho_i d/dr_i^+ p)
-    const T sx = a.asx[i], sy = a.asy[j];
+    const T sx = px, sy = py;
     const T vx = sx * (sx * st.v0 - st.v2 * in0);
     const T vy = sy * (sy * st.v1 - st.v3 * in1);
     a.vx[gb + g] = vx;
@@ -133,7 +144,7 @@ __device__ __forceinline__ void row_point(const PropArgs<T>& a, const int ph, co
     // eq. num-rho with the additive source of eq. s1 (dt s_i = P0 / (2 d c^2))
     T q = (T)0;
     if ((a.flags & kSource) && interior) q = a.io->p0[(long long)b * a.n0 * a.n1 + ii] / ((T)4 * st.v3);
-    const T ax = a.ax[i], ay = a.ay[j], r0 = st.v2;
+    const T ax = px, ay = py, r0 = st.v2;
     const T rx = ax * (ax * st.v0 - a.dt * r0 * in0) + q;
     const T ry = ay * (ay * st.v1 - a.dt * r0 * in1) + q;
     a.rx[gb + g] = rx;
@@ -163,7 +174,7 @@ __device__ __forceinline__ void row_point(const PropArgs<T>& a, const int ph, co
       ya = in1;
     }
     const T rpart = (ph == A_R1L) ? Cp : Cp - in0;   // (I - Y_dis eta) C p-bar
-    const T ax = a.ax[i], ay = a.ay[j], r0 = st.v2;
+    const T ax = px, ay = py, r0 = st.v2;
     const T rtx = st.v0 + rpart;
     const T rty = st.v1 + rpart;
     out0 = r0 * ax * (ya - a.dt * rtx);
@@ -179,7 +190,7 @@ __device__ __forceinline__ void row_point(const PropArgs<T>& a, const int ph, co
     }
   } else if (ph == A_R5) {
     // transpose of the velocity update
-    const T sx = a.asx[i], sy = a.asy[j];
+    const T sx = px, sy = py;
     const T vtx = st.v0 + in0;
     const T vty = st.v1 + in1;
     a.vx[gb + g] = sx * sx * vtx;
@@ -247,6 +258,72 @@ __device__ __forceinline__ void col_point(const PropArgs<T>& a, const int ph, co
                                           const C X1, C& o0, C& o1) {
   const ColIn<T, C> st = col_load<T, C>(a, ph, kx, ky);
   col_apply<T, C>(ph, st, col_sx<T, C>(a, ph, kx), X0, X1, o0, o1);
+}
+
+// ---- what the two spectral slots hold (FP32) ---------------------------------
+// Two fields f0, f1 between passes travel as the one complex field Z = f0 + i f1
+// (kin or kout = 2): slot 0 holds Z(kx) for kx = 0 .. L/2, slot 1 conj Z(-kx) for
+// kx = 1 .. L/2 - 1, per grid row.  A row pass is then one complex transform per
+// row each way, stored straight from registers, with the two rows of a pair as
+// the lanes of the packed stream; the column pass, which has A = Z(kx) and
+// B = conj Z(-kx) of a spectral point in one thread, separates F0 = (A + B)/2,
+// F1 = (A - B)/(2i) and joins G0 + i G1, G0 - i G1.  (With a half spectrum per
+// field in each slot the row passes merged and split two rows per transform
+// through shared memory, 50.9 ms against 49.5 at 576^2 batch 12, 150 steps; the
+// FP64 passes, bound by FP64 arithmetic, still do.)  One field (kin or kout = 1: the pressure) is packed as
+// two rows of a complex transform, its half spectrum in slot 0.  Fields sharing a
+// transform are balanced by powers of two (PropArgs su .. sa).
+template <typename C>
+__device__ __forceinline__ C packed_in(const C* s0, const C* s1, int n, int L) {   // conj Z(n) of one row
+  return 2 * n <= L ? cconj(s0[n]) : s1[L - n];
+}
+template <typename C>
+__device__ __forceinline__ void packed_out(C* s0, C* s1, int n, int L, C Z) {
+  if (2 * n <= L) s0[n] = Z;
+  else s1[L - n] = cconj(Z);
+}
+// Products and sums rounded on their own, never contracted into a neighbour's
+// fused multiply-add: which of two products a compiler fuses may differ between
+// kernels, and a member of a group has the bits of its own passes.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+// Factor of the second incoming / outgoing field of a row pass and of the
+// second symbol of a column pass.
+template <typename T>
+__device__ __forceinline__ T in1_scale(const PropArgs<T>& a, int ph) { return ph == F_R1 ? a.sy : ph == A_R3 ? a.sa : (T)1; }
+template <typename T>
+__device__ __forceinline__ T out1_scale(const PropArgs<T>& a, int ph) { return ph == F_R3 ? a.su : ph == A_R1 ? a.st : (T)1; }
+template <typename T>
+__device__ __forceinline__ T k2_scale(const PropArgs<T>& a, int ph) {
+  return ph == F_C3 ? (T)1 / (a.su * a.sy) : ph == A_C2 ? (T)1 / (a.st * a.sa) : (T)1;
+}
+// Spectral products on the transforms X0, X1 of the two slots of a column.
+template <typename T, typename C>
+__device__ __forceinline__ void packed_col(const int ph, ColIn<T, C> st, const C sx, const C X0, const C X1,
+                                           C& o0, C& o1) {
+  C F0 = X0, F1 = X0, G0, G1;
+  if (col_kin(ph) == 2) {                          // (the half is in the symbols: col_half)
+    F0 = cadd(X0, X1);
+    F1 = cmul_mi(csub(X0, X1));
+  }
+  col_apply<T, C>(ph, st, sx, F0, F1, G0, G1);
+  o0 = G0;
+  o1 = G1;
+  if (col_kout(ph) == 2) {
+    o0 = cmake<C>(add_rn(G0.x, -G1.y), add_rn(G0.y, G1.x));
+    o1 = cmake<C>(add_rn(G0.x, G1.y), add_rn(G0.y, -G1.x));
+  }
+}
+// Symbols of a column point with the half of F0, F1 and the balance factor.
+template <typename T, typename C>
+__device__ __forceinline__ ColIn<T, C> col_half(const PropArgs<T>& a, const int ph, ColIn<T, C> st, const T k2s) {
+  if (col_kin(ph) == 2) {
+    st.k1 *= (T)0.5;
+    st.k2 *= (T)0.5 * k2s;
+  }
+  return st;
 }
 
 // M^T w_n for the grid points of rows j0, j0 + 1 into sc[rr * nx + i]

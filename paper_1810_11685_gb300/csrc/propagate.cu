@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(kRowThreads, generic_minb<T>()) row_kernel(con
   typedef typename V2<T>::t C;
   constexpr int KIN = RowIO<PH>::kin;
   constexpr int KOUT = RowIO<PH>::kout;
+  constexpr bool PK = sizeof(T) == 4;                  // two fields as one complex field (pass_ops.cuh)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nx = a.nx;
   C* buf0 = reinterpret_cast<C*>(smem_raw);
@@ -79,7 +80,14 @@ __global__ void __launch_bounds__(kRowThreads, generic_minb<T>()) row_kernel(con
   //    half spectra of rows j0 (A) and j0+1 (B); the unnormalised inverse
   //    z = conj(FFT(conj Z)) holds row j0 in Re z and row j0+1 in Im z.
   C* res = buf0;
-  if (!skip_in) {
+  if (PK && KIN == 2 && !skip_in) {
+    for (int s = 0; s < 2; ++s) {                      // line s: row j0 + s
+      const C* s0 = spec + (long long)(j0 + s) * a.pitch;
+      for (int k = tid; k < nx; k += nth) buf0[s * nx + k] = packed_in(s0, s0 + slot, k, nx);
+    }
+    __syncthreads();
+    res = fft_batch(a.px, buf0, buf1, 2, nx, a.twx);
+  } else if (!skip_in) {
     for (int s = 0; s < KIN; ++s) {
       const C* r0 = spec + s * slot + (long long)j0 * a.pitch;
       const C* r1 = r0 + a.pitch;
@@ -115,7 +123,11 @@ __global__ void __launch_bounds__(kRowThreads, generic_minb<T>()) row_kernel(con
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
       T in0 = (T)0, in1 = (T)0;
-      if (!skip_in) {
+      if (PK && KIN == 2 && !skip_in) {
+        const C z = res[rr * nx + i];                  // conj(f0 + i f1) of row j0 + rr
+        in0 = z.x;
+        in1 = mul_rn(-z.y, in1_scale(a, PH));
+      } else if (!skip_in) {
         // res = FFT(conj Z) = conj(z): row j0 is Re, row j0+1 is -Im
         C z0 = res[i];
         in0 = rr ? -z0.y : z0.x;
@@ -126,8 +138,11 @@ __global__ void __launch_bounds__(kRowThreads, generic_minb<T>()) row_kernel(con
       }
       const T scv = (PH == A_R1 || PH == A_R1L) ? sc[rr * nx + i] : (T)0;
       T out0, out1;
-      row_point<T>(a, PH, b, i, j0 + rr, in0, in1, scv, row_load<T>(a, PH, b, i, j0 + rr), out0, out1, bad);
-      if (rr == 0) {
+      row_point<T>(a, PH, b, i, j0 + rr, in0, in1, scv, row_load<T>(a, PH, b, i, j0 + rr),
+                   row_pml_x(a, PH, i), row_pml_y(a, PH, j0 + rr), out0, out1, bad);
+      if (PK && KOUT == 2) {
+        oth[rr * nx + i] = cmake<C>(out0, mul_rn(out1, out1_scale(a, PH)));
+      } else if (rr == 0) {
         oth[i].x = out0;
         if (KOUT > 1) oth[nx + i].x = out1;
       } else {
@@ -142,6 +157,13 @@ __global__ void __launch_bounds__(kRowThreads, generic_minb<T>()) row_kernel(con
   // 3. forward x-transform of the packed rows and split into two half spectra:
   //    A(k) = (Z(k) + conj Z(-k)) / 2, B(k) = -i (Z(k) - conj Z(-k)) / 2
   C* res2 = fft_batch(a.px, oth, res, KOUT, nx, a.twx);
+  if (PK && KOUT == 2) {
+    for (int s = 0; s < 2; ++s) {
+      C* s0 = spec + (long long)(j0 + s) * a.pitch;
+      for (int k = tid; k < nx; k += nth) packed_out(s0, s0 + slot, k, nx, res2[s * nx + k]);
+    }
+    return;
+  }
   for (int o = 0; o < KOUT; ++o) {
     C* w0 = spec + o * slot + (long long)j0 * a.pitch;
     C* w1 = w0 + a.pitch;
@@ -162,6 +184,7 @@ __global__ void __launch_bounds__(kColThreads, generic_minb<T>()) col_kernel(con
   typedef typename V2<T>::t C;
   constexpr int KIN = ColIO<PH>::kin;
   constexpr int KOUT = ColIO<PH>::kout;
+  constexpr bool PK = sizeof(T) == 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int cb = a.cb, ny = a.ny, S = ny + 1, nxh = a.nxh;
   C* buf0 = reinterpret_cast<C*>(smem_raw);
@@ -180,7 +203,8 @@ __global__ void __launch_bounds__(kColThreads, generic_minb<T>()) col_kernel(con
     for (int idx = tid; idx < ny * cb; idx += nth) {
       const int ky = by_cb.div(idx), c = idx - ky * cb, kx = kx0 + c;
       C v = cmake<C>((T)0, (T)0);
-      if (kx < nxh) v = spec[s * slot + (long long)ky * a.pitch + kx];
+      if (PK && s == 1 && (kx == 0 || 2 * kx == a.nx)) v = cconj(spec[(long long)ky * a.pitch + kx]);
+      else if (kx < nxh) v = spec[s * slot + (long long)ky * a.pitch + kx];
       buf0[(s * cb + c) * S + ky] = v;
     }
   }
@@ -188,13 +212,19 @@ __global__ void __launch_bounds__(kColThreads, generic_minb<T>()) col_kernel(con
   C* res = fft_batch(a.py, buf0, buf1, KIN * cb, S, a.twy);
   C* oth = (res == buf0) ? buf1 : buf0;
 
+  const T k2s = k2_scale(a, PH);
   for (int idx = tid; idx < ny * cb; idx += nth) {
     const int c = by_ny.div(idx), ky = idx - c * ny, kx = kx0 + c;
     C o0 = cmake<C>((T)0, (T)0), o1 = o0;
     if (kx < nxh) {
       const C X0 = res[c * S + ky];
       const C X1 = (KIN > 1) ? res[(cb + c) * S + ky] : X0;
-      col_point<T, C>(a, PH, kx, ky, X0, X1, o0, o1);
+      if (PK) {
+        packed_col<T, C>(PH, col_half<T, C>(a, PH, col_load<T, C>(a, PH, kx, ky), k2s), col_sx<T, C>(a, PH, kx), X0, X1,
+                         o0, o1);
+      } else {
+        col_point<T, C>(a, PH, kx, ky, X0, X1, o0, o1);
+      }
     }
     oth[c * S + ky] = cconj(o0);
     if (KOUT > 1) oth[(cb + c) * S + ky] = cconj(o1);

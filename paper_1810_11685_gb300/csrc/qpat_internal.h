@@ -64,6 +64,8 @@ struct PropArgs {
   FFTPlan px, py;
   const C* twx;
   const C* twy;
+  const C* twxf;          // stage twiddles of the specialised x transforms (stage_twiddles):
+  const C* twxi;          // of the plan, and of the reversed plan
   // 1: the row (x) / column (y) passes run the length-specialised kernels
   int fast_rows, fast_cols;
   // medium diagonals on the full grid [ny][nx]
@@ -79,6 +81,11 @@ struct PropArgs {
   const T* ay;
   const T* asy;
   T dt;
+  // Powers of two that balance two fields sharing a transform (FP32): with
+  // k c ~ omega and omega dt < 1, u ~ omega sum rho is sent as su u and
+  // Y_abs u ~ c k^(y-1) as Y_abs u / sy (forward), tau Cp as st tau Cp and
+  // Y_abs^T tau Cp as Y_abs^T tau Cp / sa (adjoint).
+  T su, sy, st, sa;
   // k-space symbols on the half spectrum [ny][nxh], each divided by nx*ny
   const T* kap;           // sinc(c_ref |k| dt / 2)
   const T* kp1;           // |k|^(y-1)
@@ -157,6 +164,14 @@ template <typename T>
 cudaError_t build_tables(const TableOut<T>& o, const double* d_c, const double* d_rho, const double* d_alpha_db,
                          int nx, int ny, int nxh, int pml, double dx, double dt, double c_ref, double pml_alpha,
                          double y, int lossless, cudaStream_t s);
+
+// Radices of the specialised passes of extent L (0, 0, 0: none; third 1: two stages).
+void fast_plan(int L, int q[3]);
+// Twiddles of the second and third stage of a Stockham plan q of length L at out,
+// in the order the butterflies read them: W_L^(k r L/(Ns R)) at (r - 1) Ns + k.
+constexpr int stage_twiddle_count(int q0, int q1, int q2) { return q0 * (q1 - 1) + q0 * q1 * (q2 - 1); }
+template <typename T>
+cudaError_t stage_twiddles(const int q[3], typename V2<T>::t* out, cudaStream_t s);
 
 // FP64 helpers (da.cu)
 struct DAArgs {

@@ -133,6 +133,29 @@ cudaError_t build_tables(const TableOut<T>& o, const double* d_c, const double* 
   return cudaGetLastError();
 }
 
+// One stage: W_(Ns R)^(k r) at (r - 1) Ns + k, as W_L^(k r step) of the table.
+template <typename C>
+__global__ void stage_twiddle_kernel(C* out, int L, int Ns, int R) {
+  const int u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u >= Ns * (R - 1)) return;
+  const int r = u / Ns + 1, k = u - (r - 1) * Ns;
+  double s, c;
+  sincospi(2.0 * (double)(k * r * (L / (Ns * R))) / (double)L, &s, &c);
+  out[u].x = c;
+  out[u].y = -s;
+}
+
+template <typename T>
+cudaError_t stage_twiddles(const int q[3], typename V2<T>::t* out, cudaStream_t s) {
+  typedef typename V2<T>::t C;
+  const int L = q[0] * q[1] * q[2], n2 = q[0] * (q[1] - 1), n3 = q[0] * q[1] * (q[2] - 1);
+  stage_twiddle_kernel<C><<<(n2 + 127) / 128, 128, 0, s>>>(out, L, q[0], q[1]);
+  if (n3 > 0) stage_twiddle_kernel<C><<<(n3 + 127) / 128, 128, 0, s>>>(out + n2, L, q[0] * q[1], q[2]);
+  return cudaGetLastError();
+}
+template cudaError_t stage_twiddles<float>(const int*, float2*, cudaStream_t);
+template cudaError_t stage_twiddles<double>(const int*, double2*, cudaStream_t);
+
 template cudaError_t build_tables<float>(const TableOut<float>&, const double*, const double*, const double*, int,
                                          int, int, int, double, double, double, double, double, int, cudaStream_t);
 template cudaError_t build_tables<double>(const TableOut<double>&, const double*, const double*, const double*, int,
