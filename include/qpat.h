@@ -275,7 +275,10 @@ qpat_status qpat_group_jvp(qpat_group* group, const int* batches, const double* 
  * col_block: threads per column-pass CTA, 288 or 576 (adjacent columns per
  *   CTA: col_block / 48 or col_block / 72).
  * largest_first: 1 hands the work items of the largest extent to the first
- *   CTAs.  Default {1, 144, 576, 1}. */
+ *   CTAs.  Default {1, 144, 576, 1}.
+ * The shape applies once it has been set or tuned.  Until then the members run
+ * their own launch sequences, one after the other where each fills the GPU,
+ * else as the branches of multi = 0 (the results are the same bit for bit). */
 typedef struct {
   int multi;
   int row_block;

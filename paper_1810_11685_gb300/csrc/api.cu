@@ -1275,6 +1275,7 @@ struct qpat_group {
   std::vector<cudaEvent_t> join;
   std::map<std::vector<int>, std::pair<cudaGraphExec_t, long long>> graphs;
   qpat_group_shape shape{1, 144, 576, 1};
+  bool chosen = false;         // the shape was set or tuned: group calls follow it
 };
 
 namespace {
@@ -1449,15 +1450,34 @@ long long seq_multi_adjoint(const std::vector<MMember>& mm, const qpat_group_sha
   return cnt;
 }
 
-// The launch sequence of a group call on the capture stream: one multi-problem
-// sequence when the shape asks for it and the members qualify, else each
-// member's own sequence as a parallel branch.
-long long seq_group(qpat_group* g, int dir, const int* batches, bool multi) {
-  if (multi) {
+// How a group call runs its members: one multi-problem sequence, each member's
+// own sequence as a parallel branch, or those sequences one after the other.
+enum GroupRun { kBranches = 0, kMulti = 1, kInTurn = 2 };
+
+// A set or tuned shape is followed.  Without one, members that each fill the
+// chip (a million grid points of all their problems: two rounds of the passes'
+// CTAs) run in turn, others as branches: 16 problems on each of 288^2, 432^2,
+// 576^2, 80 steps, take 30.0 ms in turn, 32.3 as branches (their working sets
+// compete for L2) and 42.4 as multi-problem launches.
+GroupRun group_run(const qpat_group* g, const int* batches) {
+  if (g->chosen) return g->shape.multi && !multi_members(g, batches).empty() ? kMulti : kBranches;
+  for (size_t i = 0; i < g->ctxs.size(); ++i)
+    if (batches[i] > 0 && (double)g->ctxs[i]->G * batches[i] < 1e6) return kBranches;
+  return kInTurn;
+}
+
+// The launch sequence of a group call on the capture stream.
+long long seq_group(qpat_group* g, int dir, const int* batches, GroupRun run) {
+  if (run == kMulti) {
     std::vector<MMember> mm = multi_members(g, batches);
     return dir == 0 ? seq_multi_forward(mm, g->shape, g->cap) : seq_multi_adjoint(mm, g->shape, g->cap);
   }
   long long kernels = 0;
+  if (run == kInTurn) {
+    for (size_t i = 0; i < g->ctxs.size(); ++i)
+      if (batches[i] > 0) kernels += seq_any(g->ctxs[i], dir, batches[i], g->cap);
+    return kernels;
+  }
   cudaEventRecord(g->fork, g->cap);
   for (size_t i = 0; i < g->ctxs.size(); ++i) {
     if (batches[i] == 0) continue;
@@ -1533,9 +1553,9 @@ qpat_status qpat_group_propagate(qpat_group* g, int dir, const int* batches, con
     if (c->prec == QPAT_FP32) set_io_for<float>(c, dir, in[i], out[i], s);
     else set_io_for<double>(c, dir, in[i], out[i], s);
   }
-  const bool multi = g->shape.multi && !multi_members(g, batches).empty();
-  key.push_back(multi ? 1 : 0);
-  if (multi) {
+  const GroupRun run = group_run(g, batches);
+  key.push_back(run);
+  if (run == kMulti) {
     key.push_back(g->shape.row_block);
     key.push_back(g->shape.col_block);
     key.push_back(g->shape.largest_first);
@@ -1545,7 +1565,7 @@ qpat_status qpat_group_propagate(qpat_group* g, int dir, const int* batches, con
     qpat_ctx* c0 = g->ctxs[0];
     cudaError_t e = cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(c0, e, "group capture");
-    const long long kernels = seq_group(g, dir, batches, multi);
+    const long long kernels = seq_group(g, dir, batches, run);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(g->cap, &graph);
     if (e != cudaSuccess) return cuda_fail(c0, e, "group capture end");
@@ -1582,6 +1602,7 @@ qpat_status qpat_group_jvp(qpat_group* g, const int* batches, const double* cons
 qpat_status qpat_group_set_shape(qpat_group* g, const qpat_group_shape* shape) {
   if (!g || !shape || !shape_valid(*shape)) return QPAT_EINVAL;
   g->shape = *shape;
+  g->chosen = true;
   return QPAT_OK;
 }
 
@@ -1652,7 +1673,7 @@ qpat_status qpat_group_tune(qpat_group* g, const int* batches, int steps, void* 
       cudaGraph_t graph = nullptr;
       cudaError_t e = cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        seq_group(g, dir, batches, multi);
+        seq_group(g, dir, batches, multi ? kMulti : kBranches);
         e = cudaStreamEndCapture(g->cap, &graph);
       }
       if (e == cudaSuccess) e = cudaGraphInstantiate(&ex[dir], graph, 0);
@@ -1689,6 +1710,7 @@ qpat_status qpat_group_tune(qpat_group* g, const int* batches, int steps, void* 
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   g->shape = st == QPAT_OK ? cand[best_k] : keep;
+  g->chosen = g->chosen || st == QPAT_OK;
   if (best) *best = g->shape;
   if (ncand) *ncand = (int)cand.size();
   return st;

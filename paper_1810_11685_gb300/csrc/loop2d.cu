@@ -1,4 +1,8 @@
 // Host side of the whole-loop kernel (loop2d.cuh): radices, fit and launch.
+#include <map>
+#include <mutex>
+#include <tuple>
+
 #include "loop2d.h"
 
 namespace qpat {
@@ -30,13 +34,28 @@ int kernel_extent(const PropArgs<float>& a) {
     default: return 0;
   }
 }
-int occupancy(int L, int adj, int ll, int nc, size_t smem) {
+int occupancy_query(int L, int adj, int ll, int nc, size_t smem) {
   switch (L) {
 #define QPAT_LOOP_CASE(L) case L: return loop_occupancy_len<L>(adj, ll, nc, smem);
     QPAT_LOOP_EXTENTS(QPAT_LOOP_CASE)
 #undef QPAT_LOOP_CASE
     default: return 0;
   }
+}
+// The query takes about a millisecond, a context creation several; its answer
+// depends on nothing but the arguments and the device.
+int occupancy(int L, int adj, int ll, int nc, size_t smem) {
+  static std::mutex mtx;
+  static std::map<std::tuple<int, int, int, int, int, size_t>, int> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const std::tuple<int, int, int, int, int, size_t> key(dev, L, adj, ll, nc, smem);
+  std::lock_guard<std::mutex> lock(mtx);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  const int n = occupancy_query(L, adj, ll, nc, smem);
+  if (n > 0) known[key] = n;
+  return n;
 }
 }  // namespace
 
