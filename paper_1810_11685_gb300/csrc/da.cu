@@ -592,99 +592,177 @@ static size_t small_smem(const SmallLevels& S) {
   for (int l = 0; l < S.n; ++l) t += (size_t)S.lev[l].N * 8;
   return t * sizeof(double);
 }
+// A level in shared memory: x and a second buffer t, b, d, w, and the face
+// coefficients cx, cy, cz.
 struct SmallLev {
   double *x, *t, *b, *d, *w, *cx, *cy, *cz;
 };
-__device__ __forceinline__ double small_res(const LevDev& L, const SmallLev& s, const double* x, int g, bool dim3_) {
+// Cell g with the offsets of its neighbours and their coefficients' (an absent
+// neighbour reads the cell itself with coefficient 0), worked out once per cell
+// and level: the sweeps have no index arithmetic left.
+struct SmallCell {
+  double cl, cr, cd, cu, cb, cf, d, w, b;
+  int il, ir, id, iu, ib, jf;
+};
+template <int DIM>
+__device__ __forceinline__ SmallCell small_cell(const LevDev& L, const SmallLev& s, int g) {
   const int sy = L.n0, sz = L.n0 * L.n1;
-  const int k = g / sz, rem = g - k * sz, j = rem / L.n0, i = rem - j * L.n0;
-  double r = s.b[g] - s.d[g] * x[g];
-  if (i > 0) r += s.cx[g - 1] * x[g - 1];
-  if (i < L.n0 - 1) r += s.cx[g] * x[g + 1];
-  if (j > 0) r += s.cy[g - sy] * x[g - sy];
-  if (j < L.n1 - 1) r += s.cy[g] * x[g + sy];
-  if (dim3_) {
-    if (k > 0) r += s.cz[g - sz] * x[g - sz];
-    if (k < L.n2 - 1) r += s.cz[g] * x[g + sz];
+  const int k = DIM == 3 ? g / sz : 0, rem = g - k * sz, j = rem / L.n0, i = rem - j * L.n0;
+  SmallCell c;
+  c.il = i > 0 ? g - 1 : g;
+  c.cl = i > 0 ? s.cx[g - 1] : 0.0;
+  c.ir = i < L.n0 - 1 ? g + 1 : g;
+  c.cr = i < L.n0 - 1 ? s.cx[g] : 0.0;
+  c.id = j > 0 ? g - sy : g;
+  c.cd = j > 0 ? s.cy[g - sy] : 0.0;
+  c.iu = j < L.n1 - 1 ? g + sy : g;
+  c.cu = j < L.n1 - 1 ? s.cy[g] : 0.0;
+  if (DIM == 3) {
+    c.ib = k > 0 ? g - sz : g;
+    c.cb = k > 0 ? s.cz[g - sz] : 0.0;
+    c.jf = k < L.n2 - 1 ? g + sz : g;
+    c.cf = k < L.n2 - 1 ? s.cz[g] : 0.0;
   }
-  return r;
+  c.d = s.d[g];
+  c.w = s.w[g];
+  c.b = s.b[g];
+  return c;
 }
-__global__ void __launch_bounds__(kThreads) mg_small(const __grid_constant__ SmallLevels S, PCGWork w) {
-  extern __shared__ __align__(16) double sm[];
-  if (w.scal[8 * blockIdx.x + 5] != 0.0) return;
-  const bool d3 = S.dim == 3;
-  const int tid = threadIdx.x;
-  SmallLev sl[kMaxSmall];
-  {
-    double* p = sm;
-#pragma unroll
-    for (int l = 0; l < kMaxSmall; ++l) {
-      if (l >= S.n) break;
-      const LevDev& L = S.lev[l];
-      const long long o = (long long)blockIdx.x * L.N;
-      sl[l] = SmallLev{p, p + L.N, p + 2 * L.N, p + 3 * L.N, p + 4 * L.N, p + 5 * L.N, p + 6 * L.N, p + 7 * L.N};
-      p += 8 * L.N;
-      for (int g = tid; g < L.N; g += kThreads) {
-        if (l == 0) sl[l].b[g] = L.b[o + g];
-        sl[l].d[g] = L.d[o + g];
-        sl[l].w[g] = L.w[o + g];
-        sl[l].cx[g] = L.cx[g];
-        sl[l].cy[g] = L.cy[g];
-        if (d3) sl[l].cz[g] = L.cz[g];
-      }
-    }
+// b - A x at cell g, as two chains of fused multiply-adds.
+template <int DIM>
+__device__ __forceinline__ double small_res(const SmallCell& c, const double* x, int g) {
+  double r = c.b - c.d * x[g];
+  double u = c.cd * x[c.id] + c.cu * x[c.iu];
+  r += c.cl * x[c.il];
+  r += c.cr * x[c.ir];
+  if (DIM == 3) {
+    u += c.cb * x[c.ib];
+    u += c.cf * x[c.jf];
   }
-  __syncthreads();
-  auto sweep = [&](int l, const double* in, double* out) {
-    const LevDev& L = S.lev[l];
-    for (int g = tid; g < L.N; g += kThreads) out[g] = in[g] + sl[l].w[g] * small_res(L, sl[l], in, g, d3);
-    __syncthreads();
-  };
+  return r + u;
+}
+// The cells of this thread on one level (kSmallCells / kThreads of them).
+constexpr int kSmallPer = (kSmallCells + kThreads - 1) / kThreads;
+template <int DIM>
+struct SmallCells {
+  SmallCell c[kSmallPer];
+  int N;
+  __device__ __forceinline__ SmallCells(const LevDev& L, const SmallLev& s) : N(L.N) {
+    each([&](int q, int g) { c[q] = small_cell<DIM>(L, s, g); });
+  }
+  template <class F>
+  __device__ __forceinline__ void each(F&& f) {
 #pragma unroll
-  for (int l = 0; l < kMaxSmall; ++l) {
-    if (l >= S.n) break;
-    const LevDev& L = S.lev[l];
-    double* first = l + 1 < S.n ? sl[l].t : sl[l].x;
-    for (int g = tid; g < L.N; g += kThreads) first[g] = sl[l].w[g] * sl[l].b[g];
+    for (int q = 0; q < kSmallPer; ++q)
+      if ((int)threadIdx.x + q * kThreads < N) f(q, (int)threadIdx.x + q * kThreads);
+  }
+  __device__ __forceinline__ void sweep(const double* in, double* out) {
+    each([&](int q, int g) { out[g] = in[g] + c[q].w * small_res<DIM>(c[q], in, g); });
     __syncthreads();
-    if (l + 1 == S.n) {
-      for (int q = 1; q < S.sweeps; q += 2) {                    // (an odd number: the result ends in x)
-        sweep(l, sl[l].x, sl[l].t);
-        sweep(l, sl[l].t, sl[l].x);
-      }
-      break;
-    }
-    sweep(l, sl[l].t, sl[l].x);
-    const LevDev& C = S.lev[l + 1];
+  }
+};
+// The V-cycle over the levels of S (b of the first is set), x of the first
+// receiving the result.
+template <int DIM>
+__device__ __forceinline__ void small_cycle(const SmallLevels& S, const SmallLev* sl) {
+  const int tid = threadIdx.x;
+  for (int l = 0; l + 1 < S.n; ++l) {
+    const LevDev &L = S.lev[l], &C = S.lev[l + 1];
+    const SmallLev s = sl[l];
+    SmallCells<DIM> c(L, s);
+    c.each([&](int q, int g) { s.t[g] = c.c[q].w * c.c[q].b; });
+    __syncthreads();
+    c.sweep(s.t, s.x);
+    // the residual of every cell, then its sum over the children of each coarse cell
+    c.each([&](int q, int g) { s.t[g] = small_res<DIM>(c.c[q], s.x, g); });
+    __syncthreads();
     for (int t = tid; t < C.N; t += kThreads) {
-      const int K = t / (C.n0 * C.n1), rem = t - K * C.n0 * C.n1, J = rem / C.n0, I = rem - J * C.n0;
+      const int K = DIM == 3 ? t / (C.n0 * C.n1) : 0, rem = t - K * C.n0 * C.n1, J = rem / C.n0, I = rem - J * C.n0;
       double acc = 0.0;
-      for (int dz = 0; dz < (d3 ? 2 : 1); ++dz)
-        for (int dy = 0; dy < 2; ++dy)
-          for (int dx = 0; dx < 2; ++dx)
-            acc += small_res(L, sl[l], sl[l].x, ((d3 ? 2 * K + dz : 0) * L.n1 + 2 * J + dy) * L.n0 + 2 * I + dx, d3);
+      for (int dz = 0; dz < (DIM == 3 ? 2 : 1); ++dz)
+        for (int dy = 0; dy < 2; ++dy) {
+          const double* f = s.t + ((DIM == 3 ? 2 * K + dz : 0) * L.n1 + 2 * J + dy) * L.n0 + 2 * I;
+          acc += f[0] + f[1];
+        }
       sl[l + 1].b[t] = acc;
     }
     __syncthreads();
   }
-#pragma unroll
-  for (int l = kMaxSmall - 2; l >= 0; --l) {
-    if (l + 1 >= S.n) continue;
-    const LevDev &L = S.lev[l], &C = S.lev[l + 1];
-    for (int g = tid; g < L.N; g += kThreads) {
-      const int k = g / (L.n0 * L.n1), rem = g - k * L.n0 * L.n1, j = rem / L.n0, i = rem - j * L.n0;
-      sl[l].x[g] += sl[l + 1].x[((d3 ? k >> 1 : 0) * C.n1 + (j >> 1)) * C.n0 + (i >> 1)];
-    }
+  {
+    // the coarsest level: an odd number of sweeps from zero, the result in x; a
+    // level of at most 32 cells stays in one warp
+    const LevDev& L = S.lev[S.n - 1];
+    const SmallLev s = sl[S.n - 1];
+    SmallCells<DIM> c(L, s);
+    c.each([&](int q, int g) { s.x[g] = c.c[q].w * c.c[q].b; });
     __syncthreads();
-    sweep(l, sl[l].x, sl[l].t);
-    sweep(l, sl[l].t, sl[l].x);
+    if (L.N > 32) {
+      for (int q = 1; q < S.sweeps; q += 2) {
+        c.sweep(s.x, s.t);
+        c.sweep(s.t, s.x);
+      }
+    } else {
+      if (tid < 32) {
+        for (int q = 1; q < S.sweeps; q += 2) {
+          if (tid < L.N) s.t[tid] = s.x[tid] + c.c[0].w * small_res<DIM>(c.c[0], s.x, tid);
+          __syncwarp();
+          if (tid < L.N) s.x[tid] = s.t[tid] + c.c[0].w * small_res<DIM>(c.c[0], s.t, tid);
+          __syncwarp();
+        }
+      }
+      __syncthreads();
+    }
   }
+  for (int l = S.n - 2; l >= 0; --l) {
+    const LevDev &L = S.lev[l], &C = S.lev[l + 1];
+    const SmallLev s = sl[l];
+    const double* xc = sl[l + 1].x;
+    SmallCells<DIM> c(L, s);
+    c.each([&](int, int g) {
+      const int k = DIM == 3 ? g / (L.n0 * L.n1) : 0, rem = g - k * L.n0 * L.n1, j = rem / L.n0, i = rem - j * L.n0;
+      s.x[g] += xc[((DIM == 3 ? k >> 1 : 0) * C.n1 + (j >> 1)) * C.n0 + (i >> 1)];
+    });
+    __syncthreads();
+    c.sweep(s.x, s.t);
+    c.sweep(s.t, s.x);
+  }
+}
+template <int DIM>
+__global__ void __launch_bounds__(kThreads) mg_small(const __grid_constant__ SmallLevels S, PCGWork w) {
+  extern __shared__ __align__(16) double sm[];
+  if (w.scal[8 * blockIdx.x + 5] != 0.0) return;
+  const int tid = threadIdx.x;
+  __shared__ SmallLev sl[kMaxSmall];
+  if (tid == 0) {
+    double* p = sm;
+    for (int l = 0; l < S.n; ++l) {
+      const int N = S.lev[l].N;
+      sl[l] = SmallLev{p, p + N, p + 2 * N, p + 3 * N, p + 4 * N, p + 5 * N, p + 6 * N, p + 7 * N};
+      p += 8 * N;
+    }
+  }
+  __syncthreads();
+  for (int l = 0; l < S.n; ++l) {
+    const LevDev& L = S.lev[l];
+    const SmallLev s = sl[l];
+    const long long o = (long long)blockIdx.x * L.N;
+    for (int g = tid; g < L.N; g += kThreads) {
+      if (l == 0) s.b[g] = L.b[o + g];
+      s.d[g] = L.d[o + g];
+      s.w[g] = L.w[o + g];
+      s.cx[g] = L.cx[g];
+      s.cy[g] = L.cy[g];
+      if (DIM == 3) s.cz[g] = L.cz[g];
+    }
+  }
+  __syncthreads();
+  small_cycle<DIM>(S, sl);
   const LevDev& L = S.lev[0];
-  const int f0 = 2 * L.n0, f1 = 2 * L.n1, Nf = L.N * (d3 ? 8 : 4);
+  const int f0 = 2 * L.n0, f1 = 2 * L.n1, Nf = L.N * (DIM == 3 ? 8 : 4);
   double* f = S.xf + (long long)blockIdx.x * Nf;
   for (int g = tid; g < Nf; g += kThreads) {
     const int k = g / (f0 * f1), rem = g - k * f0 * f1, j = rem / f0, i = rem - j * f0;
-    f[g] += sl[0].x[((d3 ? k >> 1 : 0) * L.n1 + (j >> 1)) * L.n0 + (i >> 1)];
+    f[g] += sl[0].x[((DIM == 3 ? k >> 1 : 0) * L.n1 + (j >> 1)) * L.n0 + (i >> 1)];
   }
 }
 
@@ -769,7 +847,8 @@ static void mg_vcycle(MGHierarchy& h, PCGWork& w, int batch, int slot, cudaStrea
     S.sweeps = h.coarse_sweeps;
     for (int l = ls; l < h.nlev; ++l) S.lev[l - ls] = mg_dev(h.lev[l], w);
     S.xf = xf;
-    mg_small<<<batch, kThreads, small_smem(S), s>>>(S, w);
+    if (dim == 3) mg_small<3><<<batch, kThreads, small_smem(S), s>>>(S, w);
+    else mg_small<2><<<batch, kThreads, small_smem(S), s>>>(S, w);
   } else if (B.A.N <= kClusterCells) {
     mg_coarse_cluster<<<kCoarseCluster * batch, kCoarseThreads, 0, s>>>(mg_dev(B, w), xf, w, dim, h.coarse_sweeps);
   } else {
