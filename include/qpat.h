@@ -221,9 +221,12 @@ qpat_status qpat_acoustic_resume(qpat_ctx* ctx, int batch, const void* ckpt, int
  * [ny][nx] (either may be NULL: not returned).  Workspace is allocated per
  * call: the tangent needs 27 real grid fields of the context precision, one
  * FP64 and 8 complex; the gradient up to 24 real of the context precision,
- * 7 to 9 FP64 and 8 complex, plus a tape of 5 (lossless) or 7 real grid
+ * 7 to 9 FP64 and 8 complex (FP64 contexts: 17 real, as much as the context's
+ * spectral workspace of one problem, and one series), plus a tape of 5
+ * (lossless) or 7 real grid
  * fields per stored time step.  The gradient keeps the tape of every step
- * while that history fits in 2 GiB; beyond, it stores the loop state (5 real grid fields) every K steps
+ * while that history fits in 2 GiB; beyond, it stores the loop state (5 real grid fields; FP64
+ * contexts: a qpat_acoustic_forward_ckpt checkpoint) every K steps
  * during the forward sweep and recomputes each segment's tape from its
  * checkpoint before the segment's transposed steps (K tape slots; K near
  * sqrt(5 nt / fields), or as set by qpat_set_medium_checkpoints).  The

@@ -58,8 +58,56 @@ size_t col_smem_bytes(int ny, int cb) {
 // ---------------------------------------------------------------------------
 // Row pass: rows j0 = 2*blockIdx.x and j0 + 1 of problem blockIdx.y.
 // ---------------------------------------------------------------------------
-template <typename T, int PH>
-__global__ void __launch_bounds__(kRowThreads, generic_minb<T>()) row_kernel(const PropArgs<T> a) {
+// Tap: NoTap, or MediumTap where the medium gradient also keeps the fields of a
+// forward step or adds the products of a transposed one (medium_tap).
+struct NoTap {};
+template <int PH, typename T>
+__device__ __forceinline__ void medium_tap(const NoTap&, const PropArgs<T>&, long long, T, T, T, const RowIn<T>&, T, T,
+                                           T) {}
+// in0, in1: the incoming fields; scv: M^T w; st: the operands before the update;
+// px, py: PML factors; out0: the first outgoing field.
+template <int PH>
+__device__ __forceinline__ void medium_tap(const MediumTap& t, const PropArgs<double>& a, long long g, double in0,
+                                           double in1, double scv, const RowIn<double>& st, double px, double py,
+                                           double out0) {
+  if (PH == F_R1) {
+    t.Yr[g] = in0;
+    t.Yu[g] = in1;
+    t.X[g] = (st.v0 + st.v1 - st.v3 * in0) + st.v4 * in1;        // p / C
+  } else if (PH == F_R2) {
+    t.gx[g] = in0;
+    t.gy[g] = in1;
+  } else if (PH == F_R3 || PH == F_R3L) {
+    t.dx[g] = in0;
+    t.dy[g] = in1;
+    if (PH == F_R3L) t.X[g] = out0 / st.v3;
+  } else if (PH == A_R5) {
+    t.grsx[g] += (st.v0 + in0) * px * st.v2 * st.v2 / a.dt * t.gx[g];
+    t.grsy[g] += (st.v1 + in1) * py * st.v3 * st.v3 / a.dt * t.gy[g];
+  } else {
+    double rpart, ya = 0.0;
+    if (PH == A_R3) {
+      rpart = st.v4 - in0;
+      ya = in1;
+    } else {
+      const double pb = in0 + scv, cp = (PH == A_R1 ? st.v2 : st.v3) * pb;
+      t.gC[g] += pb * t.X[g];
+      if (PH == A_R1) {
+        t.geta[g] -= cp * t.Yr[g];
+        t.gtau[g] += cp * t.Yu[g];
+        return;
+      }
+      rpart = cp;
+    }
+    const double tx = st.v0 + rpart, ty = st.v1 + rpart;
+    t.grho[g] += px * t.dx[g] * (ya - a.dt * tx) + py * t.dy[g] * (ya - a.dt * ty);
+    if (t.qb) t.qb[g] += tx + ty;
+  }
+}
+
+template <typename T, int PH, typename Tap = NoTap>
+__global__ void __launch_bounds__(kRowThreads, std::is_same<Tap, NoTap>::value ? generic_minb<T>() : 2)
+row_kernel(const PropArgs<T> a, const Tap tap = Tap{}) {
   typedef typename V2<T>::t C;
   constexpr int KIN = RowIO<PH>::kin;
   constexpr int KOUT = RowIO<PH>::kout;
@@ -138,8 +186,10 @@ __global__ void __launch_bounds__(kRowThreads, generic_minb<T>()) row_kernel(con
       }
       const T scv = (PH == A_R1 || PH == A_R1L) ? sc[rr * nx + i] : (T)0;
       T out0, out1;
-      row_point<T>(a, PH, b, i, j0 + rr, in0, in1, scv, row_load<T>(a, PH, b, i, j0 + rr),
-                   row_pml_x(a, PH, i), row_pml_y(a, PH, j0 + rr), out0, out1, bad);
+      const RowIn<T> st = row_load<T>(a, PH, b, i, j0 + rr);
+      const T px = row_pml_x(a, PH, i), py = row_pml_y(a, PH, j0 + rr);
+      row_point<T>(a, PH, b, i, j0 + rr, in0, in1, scv, st, px, py, out0, out1, bad);
+      medium_tap<PH>(tap, a, (long long)(j0 + rr) * nx + i, in0, in1, scv, st, px, py, out0);
       if (PK && KOUT == 2) {
         oth[rr * nx + i] = cmake<C>(out0, mul_rn(out1, out1_scale(a, PH)));
       } else if (rr == 0) {
@@ -303,14 +353,14 @@ void launch_row(const PropArgs<T>& a, int phase, int batch, cudaStream_t s) {
   dim3 grid(a.ny / 2, batch);
   const size_t sm = row_smem_bytes<T>(a.nx);
   switch (phase) {
-    case F_R1: row_kernel<T, F_R1><<<grid, kRowThreads, sm, s>>>(a); break;
-    case F_R2: row_kernel<T, F_R2><<<grid, kRowThreads, sm, s>>>(a); break;
-    case F_R3: row_kernel<T, F_R3><<<grid, kRowThreads, sm, s>>>(a); break;
-    case F_R3L: row_kernel<T, F_R3L><<<grid, kRowThreads, sm, s>>>(a); break;
-    case A_R1: row_kernel<T, A_R1><<<grid, kRowThreads, sm, s>>>(a); break;
-    case A_R1L: row_kernel<T, A_R1L><<<grid, kRowThreads, sm, s>>>(a); break;
-    case A_R3: row_kernel<T, A_R3><<<grid, kRowThreads, sm, s>>>(a); break;
-    case A_R5: row_kernel<T, A_R5><<<grid, kRowThreads, sm, s>>>(a); break;
+    case F_R1: row_kernel<T, F_R1><<<grid, kRowThreads, sm, s>>>(a, NoTap{}); break;
+    case F_R2: row_kernel<T, F_R2><<<grid, kRowThreads, sm, s>>>(a, NoTap{}); break;
+    case F_R3: row_kernel<T, F_R3><<<grid, kRowThreads, sm, s>>>(a, NoTap{}); break;
+    case F_R3L: row_kernel<T, F_R3L><<<grid, kRowThreads, sm, s>>>(a, NoTap{}); break;
+    case A_R1: row_kernel<T, A_R1><<<grid, kRowThreads, sm, s>>>(a, NoTap{}); break;
+    case A_R1L: row_kernel<T, A_R1L><<<grid, kRowThreads, sm, s>>>(a, NoTap{}); break;
+    case A_R3: row_kernel<T, A_R3><<<grid, kRowThreads, sm, s>>>(a, NoTap{}); break;
+    case A_R5: row_kernel<T, A_R5><<<grid, kRowThreads, sm, s>>>(a, NoTap{}); break;
     default: break;
   }
 }
@@ -333,6 +383,25 @@ static int col_width(int cb, int nxh, int batch) {
 static int col_threads(int ny, int cb) {
   const int t = (cb * ny + 31) / 32 * 32;
   return t < 64 ? 64 : t > kColThreads ? kColThreads : t;
+}
+
+void launch_row_tap(const PropArgs<double>& a, int phase, const MediumTap& tap, cudaStream_t s) {
+  const dim3 grid(a.ny / 2, 1);
+  const size_t sm = row_smem_bytes<double>(a.nx);
+  switch (phase) {
+#define QPAT_TAP_CASE(PH) case PH: row_kernel<double, PH, MediumTap><<<grid, kRowThreads, sm, s>>>(a, tap); break;
+    QPAT_TAP_CASE(F_R1) QPAT_TAP_CASE(F_R2) QPAT_TAP_CASE(F_R3) QPAT_TAP_CASE(F_R3L)
+    QPAT_TAP_CASE(A_R1) QPAT_TAP_CASE(A_R1L) QPAT_TAP_CASE(A_R3) QPAT_TAP_CASE(A_R5)
+#undef QPAT_TAP_CASE
+    default: break;
+  }
+}
+void init_row_tap() {
+#define QPAT_TAP_ATTR(PH) \
+  cudaFuncSetAttribute(row_kernel<double, PH, MediumTap>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  QPAT_TAP_ATTR(F_R1) QPAT_TAP_ATTR(F_R2) QPAT_TAP_ATTR(F_R3) QPAT_TAP_ATTR(F_R3L)
+  QPAT_TAP_ATTR(A_R1) QPAT_TAP_ATTR(A_R1L) QPAT_TAP_ATTR(A_R3) QPAT_TAP_ATTR(A_R5)
+#undef QPAT_TAP_ATTR
 }
 
 template <typename T>

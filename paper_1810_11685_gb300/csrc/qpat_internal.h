@@ -117,8 +117,20 @@ struct PropArgs {
   int* err;               // device flags word (bit 0: non-finite; bit 1: a bounded wait gave up)
 };
 
+// What the row passes of the FP64 medium gradient keep and add up, all [ny][nx]:
+// the fields of one forward step (g_i = D+_i p, the divergences, X = p / C, Y_dis
+// sum rho, Y_abs u), and the sums over the transposed steps (qb: the source
+// adjoint, null except at the source steps).
+struct MediumTap {
+  double *gx, *gy, *dx, *dy, *X, *Yr, *Yu;
+  double *gC, *geta, *gtau, *grho, *grsx, *grsy, *qb;
+};
 template <typename T>
 void launch_row(const PropArgs<T>& a, int phase, int batch, cudaStream_t s);
+// The row pass of one FP64 problem with its medium tap; init_row_tap sets the
+// kernels' attributes.
+void launch_row_tap(const PropArgs<double>& a, int phase, const MediumTap& tap, cudaStream_t s);
+void init_row_tap();
 template <typename T>
 void launch_col(const PropArgs<T>& a, int phase, int batch, cudaStream_t s);
 template <typename T>
