@@ -282,16 +282,21 @@ cudaError_t mg_setup(MGHierarchy& h, const DAArgs& fine, const double* d_kappa, 
     ++h.nlev;
   }
   for (int l = 0; l < h.nlev; ++l) {
+    // one allocation a level (each takes some tenths of a millisecond); level 0
+    // uses the PCG work vectors but for x2
     MGLevel& L = h.lev[l];
-    const size_t bytes = (size_t)max_batch * L.A.N * sizeof(double);
-    cudaError_t e;
-    if (l > 0 && (e = alloc(owner, (void**)&L.mu, bytes)) != cudaSuccess) return e;
-    if ((e = alloc(owner, (void**)&L.x2, bytes)) != cudaSuccess) return e;
-    if (l > 0 && (e = alloc(owner, (void**)&L.x, bytes)) != cudaSuccess) return e;
-    if (l > 0 && (e = alloc(owner, (void**)&L.b, bytes)) != cudaSuccess) return e;
-    // (level 0 uses the PCG work vectors for these)
-    if (l > 0 && (e = alloc(owner, (void**)&L.d, bytes)) != cudaSuccess) return e;
-    if (l > 0 && (e = alloc(owner, (void**)&L.w, bytes)) != cudaSuccess) return e;
+    const size_t n = ((size_t)max_batch * L.A.N + 1) & ~(size_t)1;   // 16-byte multiples
+    double* v = nullptr;
+    const cudaError_t e = alloc(owner, (void**)&v, (l > 0 ? 6 : 1) * n * sizeof(double));
+    if (e != cudaSuccess) return e;
+    L.x2 = v;
+    if (l > 0) {
+      L.mu = v + n;
+      L.x = v + 2 * n;
+      L.b = v + 3 * n;
+      L.d = v + 4 * n;
+      L.w = v + 5 * n;
+    }
   }
   return cudaGetLastError();
 }
