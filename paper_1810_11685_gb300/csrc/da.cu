@@ -8,8 +8,9 @@
 // gradient, adds 2 gamma kappa h / (gamma h + kappa) to the diagonal and
 // 2 kappa I h / (gamma h + kappa) to the right-hand side per boundary face;
 // absorption adds mu h^2.  The matrix is symmetric positive definite and is
-// solved by Jacobi-preconditioned conjugate gradients with FP64 dot products
-// (deterministic two-level reductions), batched over problems.
+// solved by conjugate gradients preconditioned with one multigrid V-cycle (or the
+// diagonal), with FP64 dot products (deterministic two-level reductions), batched
+// over problems.
 #include <algorithm>
 
 #include "qpat_internal.h"

@@ -6,7 +6,8 @@
 // in its precision (FP64 or FP32; directions, weights, outputs and gradient
 // sums FP64).  Every per-element functor is launched as a grid-stride kernel on
 // the context's stream; 2D FFTs run as one shared-memory line-FFT launch per
-// axis.
+// axis.  The FP64 gradient runs on the context's propagation passes instead
+// (vjp_medium_passes).
 #include <math.h>
 
 #include <map>

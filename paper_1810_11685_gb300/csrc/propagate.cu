@@ -4,11 +4,12 @@
 // num-p, num-m) and of its exact transpose (Section 3.2.4, Lemma 2) is a
 // chain of alternating passes over the 2D FFT grid:
 //
-//   row pass    : inverse x-FFT of the incoming half spectra (two grid rows
-//                 packed into one complex transform), the pointwise PML /
-//                 medium update of eqs. num-vel / num-rho / num-p, and the
-//                 forward x-FFT of the outgoing fields (again two rows per
-//                 complex transform), all in shared memory;
+//   row pass    : inverse x-FFT of the incoming spectra (FP64, and single
+//                 fields in FP32: two grid rows packed into one complex
+//                 transform; two fields in FP32: one complex transform per row,
+//                 see pass_ops.cuh), the pointwise PML / medium update of eqs.
+//                 num-vel / num-rho / num-p, and the forward x-FFT of the
+//                 outgoing fields, all in shared memory;
 //   column pass : forward y-FFT of a tile of half-spectrum columns, the
 //                 spectral symbol of eq. grr (i k_i e^{+-i k_i dx/2} kappa) or
 //                 of the fractional Laplacians Y_dis / Y_abs, and the inverse

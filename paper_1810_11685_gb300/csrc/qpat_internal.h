@@ -225,8 +225,8 @@ struct PCGWork {
   double *scal;                            // [B][8]
   double *hostscal;                        // pinned [B][8]
   MGHierarchy* mg;                         // null: Jacobi preconditioner
-  double* mu;                              // [B][N] copy of the absorption of the current solve
-  // CUDA graph of kPCGChunk iterations (fixed pointers: mu is staged in `mu`)
+  double* mu;                              // [B][N] copy of the absorption (diagonal preconditioner)
+  // CUDA graph of kPCGChunk iterations (fixed pointers)
   bool use_graphs;
   cudaStream_t cap;
   cudaGraphExec_t chunk;
