@@ -121,6 +121,61 @@ enum LoopIn : int { kInRow2, kInRowHalf, kInCol2, kInCol1 };
 // Last stage: where its points are written.
 enum LoopOut : int { kOutRow2, kOutRow1, kOutCol2, kOutColHalf };
 
+// Entry (row, column) of a problem's exchange buffer.
+struct LoopCell {
+  int row, col;
+};
+__host__ __device__ constexpr int loop_mirror(int kx, int nx) { return kx == 0 ? 0 : nx - kx; }
+// Entries of point i of a line (a row pair or a column) in its first and last
+// stage; `which` of the two that a packed pair takes.  The ranks of a cluster
+// meet only between passes, so a pass may write no entry that another rank reads
+// in it: a line's writes stay within the rows (the columns) that belong to it.
+// The packed pressure of rows 2 line, 2 line + 1 therefore lies in row 2 line,
+// although half the rows would hold it.
+__host__ __device__ constexpr LoopCell loop_in_cell(int kind, int line, int i, int which, int nx) {
+  return kind == kInRow2      ? LoopCell{2 * line + which, i}
+         : kind == kInRowHalf ? LoopCell{2 * line + which, 2 * i <= nx ? i : nx - i}
+                              : LoopCell{kind == kInCol1 ? i & ~1 : i, which ? loop_mirror(line, nx) : line};
+}
+__host__ __device__ constexpr LoopCell loop_out_cell(int kind, int line, int i, int which, int nx) {
+  return kind == kOutRow2   ? LoopCell{2 * line + which, i}
+         : kind == kOutRow1 ? LoopCell{2 * line, i}
+                            : LoopCell{i, which ? loop_mirror(line, nx) : line};
+}
+// Whether pass ph takes in, or leaves, one field.
+__host__ __device__ constexpr bool loop_one_in(int ph) { return ph == F_C1 || ph == A_R1 || ph == A_R1L; }
+__host__ __device__ constexpr bool loop_one_out(int ph) { return ph == F_R1 || ph == F_R3L || ph == A_C6; }
+__host__ __device__ constexpr bool loop_is_row(int ph) { return ph < 10 || (ph >= 20 && ph < 30); }
+// f(integral constant of the kind) for pass ph's first stage, and for its last.
+template <int K>
+using LoopKind = std::integral_constant<int, K>;
+#pragma nv_exec_check_disable
+template <bool ADJ, class F>
+__host__ __device__ __forceinline__ void loop_with_in(int ph, F&& f) {
+  if constexpr (!ADJ) {
+    if (loop_is_row(ph)) f(LoopKind<kInRow2>{});
+    else if (loop_one_in(ph)) f(LoopKind<kInCol1>{});
+    else f(LoopKind<kInCol2>{});
+  } else {
+    if (!loop_is_row(ph)) f(LoopKind<kInCol2>{});
+    else if (loop_one_in(ph)) f(LoopKind<kInRowHalf>{});
+    else f(LoopKind<kInRow2>{});
+  }
+}
+#pragma nv_exec_check_disable
+template <bool ADJ, class F>
+__host__ __device__ __forceinline__ void loop_with_out(int ph, F&& f) {
+  if constexpr (!ADJ) {
+    if (!loop_is_row(ph)) f(LoopKind<kOutCol2>{});
+    else if (loop_one_out(ph)) f(LoopKind<kOutRow1>{});
+    else f(LoopKind<kOutRow2>{});
+  } else {
+    if (loop_is_row(ph)) f(LoopKind<kOutRow2>{});
+    else if (loop_one_out(ph)) f(LoopKind<kOutColHalf>{});
+    else f(LoopKind<kOutCol2>{});
+  }
+}
+
 // Entry i of a line: a packed pair (16 bytes) or one complex value (8 bytes).
 __device__ __forceinline__ void put(float4* line, int i, P2 v) { line[i] = p2_bits(v); }
 __device__ __forceinline__ void put(float4* line, int i, float2 v) { reinterpret_cast<float2*>(line)[i] = v; }
@@ -148,47 +203,43 @@ __device__ __forceinline__ void gather_operands(const LoopCtx& c, const float4* 
 
 template <int KIND>
 __device__ __forceinline__ auto load_point(const LoopCtx& c, int m, int i, int L) {
-  if constexpr (KIND == kInRow2) {                               // conj of rows 2(line0 + m), + 1
-    const float2* r = c.spec + 2LL * (c.line0 + m) * c.rs + i;
-    return pack2(cconj(__ldcg(r)), cconj(__ldcg(r + c.rs)));
+  const int line = c.line0 + m;
+  auto at = [&](int which) {
+    const LoopCell q = loop_in_cell(KIND, line, i, which, c.nx);
+    return __ldcg(c.spec + (long long)q.row * c.rs + q.col);
+  };
+  if constexpr (KIND == kInRow2) {                               // conj of rows 2 line, 2 line + 1
+    return pack2(cconj(at(0)), cconj(at(1)));
   } else if constexpr (KIND == kInRowHalf) {                     // conj(P + i Q) of two rows' half spectra
-    const float2* r = c.spec + 2LL * (c.line0 + m) * c.rs;
-    const bool lo = 2 * i <= L;
-    const int k = lo ? i : L - i;
-    float2 P = __ldcg(r + k), Q = __ldcg(r + c.rs + k);
-    if (k == 0 || 2 * k == L) { P.y = 0.f; Q.y = 0.f; }
-    if (!lo) { P.y = -P.y; Q.y = -Q.y; }
+    float2 P = at(0), Q = at(1);
+    if (i == 0 || 2 * i == L) { P.y = 0.f; Q.y = 0.f; }
+    if (2 * i > L) { P.y = -P.y; Q.y = -Q.y; }
     return make_float2(P.x - Q.y, -(P.y + Q.x));
-  } else {
-    const int kx = c.line0 + m, km = kx == 0 ? 0 : c.nx - kx;
-    if constexpr (KIND == kInCol2) {
-      const float2* r = c.spec + (long long)i * c.rs;
-      return pack2(__ldcg(r + kx), cconj(__ldcg(r + km)));
-    } else {                                                     // row i of a field packed two rows to a line
-      const float2* r = c.spec + (long long)(i >> 1) * c.rs;
-      const float2 Z = __ldcg(r + kx), Zm = cconj(__ldcg(r + km));
-      return (i & 1) ? cscale(cmul_mi(csub(Z, Zm)), 0.5f) : cscale(cadd(Z, Zm), 0.5f);
-    }
+  } else if constexpr (KIND == kInCol2) {
+    return pack2(at(0), cconj(at(1)));
+  } else {                                                       // row i of a field packed two rows to a line
+    const float2 Z = at(0), Zm = cconj(at(1));
+    return (i & 1) ? cscale(cmul_mi(csub(Z, Zm)), 0.5f) : cscale(cadd(Z, Zm), 0.5f);
   }
 }
 
 template <int KIND, typename E>
 __device__ __forceinline__ void store_point(const LoopCtx& c, int m, int i, E v) {
+  const int line = c.line0 + m;
+  auto put_at = [&](int which, float2 z) {
+    const LoopCell q = loop_out_cell(KIND, line, i, which, c.nx);
+    c.spec[(long long)q.row * c.rs + q.col] = z;
+  };
   if constexpr (KIND == kOutRow2) {
-    float2* r = c.spec + 2LL * (c.line0 + m) * c.rs + i;
-    r[0] = lane0(v);
-    r[c.rs] = lane1(v);
+    put_at(0, lane0(v));
+    put_at(1, lane1(v));
   } else if constexpr (KIND == kOutRow1) {
-    c.spec[(long long)(c.line0 + m) * c.rs + i] = v;
+    put_at(0, v);
+  } else if constexpr (KIND == kOutCol2) {
+    put_at(0, cconj(lane0(v)));
+    if (loop_mirror(line, c.nx) != line) put_at(1, lane1(v));
   } else {
-    const int kx = c.line0 + m, km = kx == 0 ? 0 : c.nx - kx;
-    float2* r = c.spec + (long long)i * c.rs;
-    if constexpr (KIND == kOutCol2) {
-      r[kx] = cconj(lane0(v));
-      if (km != kx) r[km] = lane1(v);
-    } else {
-      r[kx] = cconj(v);
-    }
+    put_at(0, cconj(v));
   }
 }
 
@@ -406,9 +457,7 @@ __device__ __forceinline__ void loop_col_point(const LoopShared& S, int ny, int 
 template <int LC, int R, int PH>
 __device__ __forceinline__ void point_stage(const LoopArgs& A, const LoopShared& S, const LoopCtx& c, const float2* tw,
                                             int b, int flags, bool& bad) {
-  constexpr bool row = PH < 10 || (PH >= 20 && PH < 30);
-  constexpr bool in1 = PH == F_C1 || PH == A_R1 || PH == A_R1L;              // one field in
-  constexpr bool out1 = PH == F_R1 || PH == F_R3L || PH == A_C6;             // one field out
+  constexpr bool row = loop_is_row(PH), in1 = loop_one_in(PH), out1 = loop_one_out(PH);
   typedef typename std::conditional<in1, float2, P2>::type Ei;
   typedef typename std::conditional<out1, float2, P2>::type Eo;
   const int L = LC ? LC : c.L, nb = L / R, tot = c.mv * nb, pitch = loop_pitch(nb);
@@ -669,7 +718,7 @@ __global__ void __launch_bounds__(loop_threads(LC), 1) loop2d_kernel(const __gri
   for (int g = A.g0; g < A.g1; ++g) {
     const LoopStep st = loop_pass<ADJ, LL>(g, A.nt);
     const int ph = st.ph, flags = st.flags;
-    const bool row = ph < 10 || (ph >= 20 && ph < 30);
+    const bool row = loop_is_row(ph);
     const LoopAxis& ax = row ? A.x : A.y;
     c.L = ax.L;
     c.q0 = ax.q[0];
@@ -696,18 +745,10 @@ __global__ void __launch_bounds__(loop_threads(LC), 1) loop2d_kernel(const __gri
     cluster_wait();
     if (!ADJ && ph == F_C1) gather(st.n);
     float4 *p0 = bufA, *p1 = bufB;
-    const bool in1 = ph == F_C1 || ph == A_R1 || ph == A_R1L, out1 = ph == F_R1 || ph == F_R3L || ph == A_C6;
+    const bool in1 = loop_one_in(ph), out1 = loop_one_out(ph);
     if (!(flags & kSkipInput)) {
       c.dst = p0;
-      if constexpr (!ADJ) {
-        if (row) first_any<LC, kInRow2>(c);
-        else if (ph == F_C1) first_any<LC, kInCol1>(c);
-        else first_any<LC, kInCol2>(c);
-      } else {
-        if (!row) first_any<LC, kInCol2>(c);
-        else if (in1) first_any<LC, kInRowHalf>(c);
-        else first_any<LC, kInRow2>(c);
-      }
+      loop_with_in<ADJ>(ph, [&](auto kind) { first_any<LC, decltype(kind)::value>(c); });
       __syncthreads();
       c.src = p0;
       c.dst = p1;
@@ -762,15 +803,7 @@ __global__ void __launch_bounds__(loop_threads(LC), 1) loop2d_kernel(const __gri
       __syncthreads();
       float4* t = p0; p0 = p1; p1 = t;
       c.src = p1;
-      if constexpr (!ADJ) {
-        if (!row) last_any<LC, kOutCol2>(c, tw.last2);
-        else if (out1) last_any<LC, kOutRow1>(c, tw.last2);
-        else last_any<LC, kOutRow2>(c, tw.last2);
-      } else {
-        if (row) last_any<LC, kOutRow2>(c, tw.last2);
-        else if (out1) last_any<LC, kOutColHalf>(c, tw.last2);
-        else last_any<LC, kOutCol2>(c, tw.last2);
-      }
+      loop_with_out<ADJ>(ph, [&](auto kind) { last_any<LC, decltype(kind)::value>(c, tw.last2); });
     }
     cluster_arrive();
   }
