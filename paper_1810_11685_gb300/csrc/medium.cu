@@ -583,13 +583,13 @@ qpat_status vjp_medium(qpat_ctx* ctx, const double* p0, const double* wts, doubl
 // checkpoint layout) and each segment's tape recomputed by the same kernels on
 // the same inputs, so the gradient is the same bit for bit for every K.
 qpat_status vjp_medium_passes(qpat_ctx* ctx, const double* p0, const double* wts, double* g_c, double* g_rho) {
+  Tables<double> t{};
+  cudaStream_t s = nullptr;
+  int st = tables_of(ctx, t, &s);                                // (refuses 3D contexts)
+  if (st != QPAT_OK) return (qpat_status)st;
   double y = 0.0;
   int ll = 0;
-  cudaStream_t s = nullptr;
   const PropArgs<double> f0 = *ctx_tables64(ctx, &y, &ll, &s);
-  Tables<double> t{};
-  int st = tables_of(ctx, t, &s);
-  if (st != QPAT_OK) return (qpat_status)st;
   init_row_tap();
   const long long G = f0.gstride;
   const int nt = f0.nt, nf = ll ? 5 : 7;
