@@ -193,8 +193,10 @@ qpat_status qpat_vjp_kappa(qpat_ctx* ctx, int batch, const double* mu, const dou
  * A checkpoint holds, per problem, v_x, v_y, rho_x, rho_y, the sampling
  * buffer and the two spectral work slots after loop iteration n with
  * (n + 1) % K == 0 (Section 3.2.3 loop), m = (n + 1)/K - 1, 0 <= m < (nt-1)/K.
- * (The work slots' layout belongs to the kernels the context runs: resume a
- * checkpoint on the context, and at the batch, that wrote it.)
+ * The form is the same for every kernel that a propagation of the context's
+ * precision may run: a resumed series has the stored one's bits where the same
+ * kernels run (same batch, choice of passes and profiling), and equals it to
+ * rounding otherwise, on other contexts of the same grid too.
  * qpat_ckpt_bytes: size of the checkpoint buffer for batch and K.
  * qpat_acoustic_forward_ckpt: H_a as qpat_acoustic_forward, also filling
  *   ckpt (device, caller-owned, qpat_ckpt_bytes bytes).

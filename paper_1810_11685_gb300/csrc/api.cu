@@ -613,30 +613,31 @@ bool use_loop(const qpat_ctx* c, int batch) {
 // checkpoint interval when checkpoints are stored.
 long long seq_loop_forward(qpat_ctx* c, int batch, cudaStream_t s, int K, bool store, int resume_m) {
   const int nt = c->nt, ll = c->cfg.lossless != 0, P = ll ? 4 : 6;
+  const SpecLayout layout = ll ? kSpecRows : kSpecPair;
   int g = ll ? -1 : -2;
   long long cnt = 0;
   if (resume_m >= 0) {
-    launch_ckpt_copy<float>(c->pf, batch, resume_m, 0, s);
-    g = (resume_m + 1) * K * P;
+    launch_ckpt_copy<float>(c->pf, batch, resume_m, 0, s, layout);
+    g = (resume_m + 1) * K * P - ll;             // lossless: from the pressure of the restored state on
   }
   const int end = (nt - 1) * P + (ll ? 0 : 1);
   int load = resume_m >= 0;
   if (store && K > 0)
     for (int m = 0; m < (nt - 1) / K; ++m) {
       const int g1 = (m + 1) * K * P;
-      launch_loop(c->pf, c->loop, 0, ll, batch, nt, g, g1, load, 1, 0, s);
-      launch_ckpt_copy<float>(c->pf, batch, m, 1, s);
+      launch_loop(c->pf, c->loop, 0, ll, batch, nt, g, g1, load, 1, 0, 0, s);
+      launch_ckpt_copy<float>(c->pf, batch, m, 1, s, layout);
       g = g1;
       load = 1;
       ++cnt;
     }
-  launch_loop(c->pf, c->loop, 0, ll, batch, nt, g, end, load, 0, 1, s);
+  launch_loop(c->pf, c->loop, 0, ll, batch, nt, g, end, load, 0, resume_m >= 0 && ll, 1, s);
   return cnt + 1;
 }
 
 long long seq_loop_adjoint(qpat_ctx* c, int batch, cudaStream_t s) {
   const int ll = c->cfg.lossless != 0;
-  launch_loop(c->pf, c->loop, 1, ll, batch, c->nt, 0, c->nt * (ll ? 4 : 6) - 3, 0, 0, 0, s);
+  launch_loop(c->pf, c->loop, 1, ll, batch, c->nt, 0, c->nt * (ll ? 4 : 6) - 3, 0, 0, 0, 0, s);
   return 1;
 }
 

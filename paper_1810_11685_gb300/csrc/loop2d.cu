@@ -99,7 +99,7 @@ int loop_waves(const LoopPlan& p, int batch) {
 }
 
 cudaError_t launch_loop(const PropArgs<float>& a, const LoopPlan& p, int adj, int lossless, int batch, int nt, int g0,
-                        int g1, int load, int save, int gather_last, cudaStream_t s) {
+                        int g1, int load, int save, int rebuild, int gather_last, cudaStream_t s) {
   const int k = choose(p, batch);
   if (k < 0) return cudaErrorInvalidConfiguration;
   const int nc = kClusters[k];
@@ -115,6 +115,7 @@ cudaError_t launch_loop(const PropArgs<float>& a, const LoopPlan& p, int adj, in
   A.g1 = g1;
   A.load = load;
   A.save = save;
+  A.rebuild = rebuild;
   A.gather_last = gather_last;
   const size_t smem = loop_smem(a, p.x, p.y, nc, adj, lossless);
   switch (kernel_extent(a)) {

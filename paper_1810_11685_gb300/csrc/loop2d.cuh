@@ -366,10 +366,13 @@ __device__ __forceinline__ void loop_row_point(const LoopArgs& A, const LoopShar
     }
     const F2 ax(S.ax[i]), ay(S.ay[m]), r0(S.rho[p]);
     const F2 dr = F2(r0 * F2(a.dt));
-    const F2 rx = q + ax * F2(ax * F2(S.rx[p]) - dr * f0);
-    const F2 ry = q + ay * F2(ay * F2(S.ry[p]) - dr * f1);
-    S.rx[p] = rx.v;
-    S.ry[p] = ry.v;
+    F2 rx(S.rx[p]), ry(S.ry[p]);
+    if (PH == F_R3 || !(flags & kRebuild)) {
+      rx = q + ax * F2(ax * rx - dr * f0);
+      ry = q + ay * F2(ay * ry - dr * f1);
+      S.rx[p] = rx.v;
+      S.ry[p] = ry.v;
+    }
     if constexpr (PH == F_R3) {
       o0 = rx + ry;
       const F2 ux = F2(ax * r0), uy = F2(ay * r0);
@@ -717,7 +720,7 @@ __global__ void __launch_bounds__(loop_threads(LC), 1) loop2d_kernel(const __gri
   cluster_arrive();
   for (int g = A.g0; g < A.g1; ++g) {
     const LoopStep st = loop_pass<ADJ, LL>(g, A.nt);
-    const int ph = st.ph, flags = st.flags;
+    const int ph = st.ph, flags = !ADJ && LL && A.rebuild && g == A.g0 ? kSkipInput | kRebuild : st.flags;
     const bool row = loop_is_row(ph);
     const LoopAxis& ax = row ? A.x : A.y;
     c.L = ax.L;

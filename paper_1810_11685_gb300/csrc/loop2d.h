@@ -65,6 +65,7 @@ struct LoopArgs {
   int nt;                  // samples of the loop
   int g0, g1;              // passes [g0, g1) of the loop (loop_pass)
   int load, save;          // restore the state from / leave it in the context's arrays
+  int rebuild;             // pass g0 only forms the pressure's spectrum from the restored state (F_R3L)
   int gather_last;         // gather sample nt - 1 at the end (forward)
 };
 
@@ -105,7 +106,7 @@ int loop_waves(const LoopPlan& p, int batch);
 // Passes [g0, g1) of H_a (adj = 0) or H_a^* (adj = 1) of nt samples for
 // `batch` problems.
 cudaError_t launch_loop(const PropArgs<float>& a, const LoopPlan& p, int adj, int lossless, int batch, int nt, int g0,
-                        int g1, int load, int save, int gather_last, cudaStream_t s);
+                        int g1, int load, int save, int rebuild, int gather_last, cudaStream_t s);
 // Per extent L (0: runtime lengths), instantiated in loop2d_*.cu.
 template <bool ADJ, bool LL, int L>
 cudaError_t loop_launch_one(const LoopArgs& A, int nc, int batch, size_t smem, cudaStream_t s);

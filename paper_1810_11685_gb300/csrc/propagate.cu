@@ -450,10 +450,42 @@ __host__ __device__ long long ckpt_elems(const PropArgs<T>& a) {
   return 5 * a.gstride + 2 * a.sstride;     // 5 real grids + 2 slots of complex (2 T each)
 }
 
+// The spectral part of a checkpoint, ck, from or to the whole-loop kernel's rows
+// (SpecLayout).  A pair of fields is the same complex values in either form, so
+// the copy is exact; the half spectra of a single field are separated as the
+// loop's column pass does, and not restored: the loop kernel forms them again
+// from the state (kRebuild), which gives its own bits.  The checkpoint, a caller's
+// buffer, is read and written by single values.
+template <typename T>
+__device__ void ckpt_loop_rows(const PropArgs<T>& a, T* ck, int b, int to_ckpt, SpecLayout layout) {
+  typedef typename V2<T>::t C;
+  C* spec = a.spec + (long long)b * a.sstride;
+  const long long slot = 2LL * a.ny * a.pitch;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < (long long)a.ny * a.nxh;
+       t += (long long)gridDim.x * blockDim.x) {
+    const int y = (int)(t / a.nxh), kx = (int)(t - (long long)y * a.nxh), km = kx == 0 ? 0 : a.nx - kx;
+    C* row = spec + (long long)(layout == kSpecRows ? y & ~1 : y) * 2 * a.pitch;
+    T* s0 = ck + 2 * ((long long)y * a.pitch + kx);
+    T* s1 = s0 + slot;
+    if (to_ckpt) {
+      C u = row[kx], v = cconj(row[km]);
+      if (layout == kSpecRows) {
+        u = (y & 1) ? cscale(cmul_mi(csub(u, v)), (T)0.5) : cscale(cadd(u, v), (T)0.5);
+        v = cmake<C>((T)0, (T)0);
+      }
+      s0[0] = u.x; s0[1] = u.y;
+      s1[0] = v.x; s1[1] = v.y;
+    } else if (layout == kSpecPair) {
+      row[kx] = cmake<C>(s0[0], s0[1]);
+      if (km != kx) row[km] = cmake<C>(s1[0], -s1[1]);
+    }
+  }
+}
+
 // One forward-state checkpoint: v_x, v_y, rho_x, rho_y, the sampling buffer
 // and both spectral slots of every problem, at checkpoint index m.
 template <typename T>
-__global__ void ckpt_copy_kernel(const PropArgs<T> a, int batch, int m, int to_ckpt) {
+__global__ void ckpt_copy_kernel(const PropArgs<T> a, int batch, int m, int to_ckpt, SpecLayout layout) {
   const int b = blockIdx.y;
   const long long per = ckpt_elems(a);
   T* ck = a.io->ckpt + ((long long)m * batch + b) * per;
@@ -463,6 +495,10 @@ __global__ void ckpt_copy_kernel(const PropArgs<T> a, int batch, int m, int to_c
   const long long len[6] = {G, G, G, G, G, 2 * a.sstride};
   long long off = 0;
   for (int f = 0; f < 6; ++f) {
+    if (f == 5 && layout != kSpecSlots) {
+      ckpt_loop_rows<T>(a, ck + off, b, to_ckpt, layout);
+      return;
+    }
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < len[f];
          t += (long long)gridDim.x * blockDim.x) {
       if (to_ckpt) ck[off + t] = src[f][t];
@@ -473,8 +509,8 @@ __global__ void ckpt_copy_kernel(const PropArgs<T> a, int batch, int m, int to_c
 }
 
 template <typename T>
-void launch_ckpt_copy(const PropArgs<T>& a, int batch, int m, int to_ckpt, cudaStream_t s) {
-  ckpt_copy_kernel<T><<<dim3(128, batch), 256, 0, s>>>(a, batch, m, to_ckpt);
+void launch_ckpt_copy(const PropArgs<T>& a, int batch, int m, int to_ckpt, cudaStream_t s, SpecLayout layout) {
+  ckpt_copy_kernel<T><<<dim3(128, batch), 256, 0, s>>>(a, batch, m, to_ckpt, layout);
 }
 
 template <typename T>
@@ -492,7 +528,7 @@ void launch_gather(const PropArgs<T>& a, int batch, cudaStream_t s) {
   template void launch_gather<T>(const PropArgs<T>&, int, cudaStream_t);                \
   template void launch_set_io<T>(IoPtrs<T>*, const T*, T*, const T*, T*, T*, cudaStream_t);  \
   template long long ckpt_elems<T>(const PropArgs<T>&);                                       \
-  template void launch_ckpt_copy<T>(const PropArgs<T>&, int, int, int, cudaStream_t);
+  template void launch_ckpt_copy<T>(const PropArgs<T>&, int, int, int, cudaStream_t, SpecLayout);
 QPAT_INST(float)
 QPAT_INST(double)
 

@@ -25,6 +25,7 @@ enum : int {
   kAccWrite = 4,     // adjoint: write the source adjoint into p0_adj
   kAccAdd = 8,       // adjoint: add the source adjoint into p0_adj
   kSkipOutput = 16,  // no outgoing spectral slots needed (last step)
+  kRebuild = 32,     // F_R3L of the whole-loop kernel: the pressure of a restored state, no update
 };
 
 // Propagation phases.  F_*: forward step (Section 3.2.3), A_*: transposed
@@ -141,9 +142,14 @@ void launch_set_io(IoPtrs<T>* dst, const T* p0, T* data, const T* w, T* p0adj, T
 // rho_x, rho_y and the sampling buffer (5 grids) plus the two spectral slots.
 template <typename T>
 __host__ __device__ long long ckpt_elems(const PropArgs<T>& a);
-// store (to_ckpt = 1) or restore the state of all problems at checkpoint m
+// What the spectral buffer holds at a checkpoint: the two slots of the launched
+// passes (pass_ops.cuh), or the whole-loop kernel's rows, of a packed pair of
+// fields or of one field packed two rows to a line (loop2d.cuh).
+enum SpecLayout : int { kSpecSlots, kSpecPair, kSpecRows };
+// store (to_ckpt = 1) or restore the state of all problems at checkpoint m;
+// a checkpoint holds slots, whatever the layout of the buffer
 template <typename T>
-void launch_ckpt_copy(const PropArgs<T>& a, int batch, int m, int to_ckpt, cudaStream_t s);
+void launch_ckpt_copy(const PropArgs<T>& a, int batch, int m, int to_ckpt, cudaStream_t s, SpecLayout layout = kSpecSlots);
 // length-specialised passes (fast_kernels.cuh), one translation unit per length
 template <typename T, int L>
 void launch_row_fast_len(const PropArgs<T>& a, int ph, int batch, cudaStream_t s);
