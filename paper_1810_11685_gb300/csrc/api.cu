@@ -64,6 +64,7 @@ struct qpat_ctx {
   size_t prof_used = 0;
   LoopPlan loop;               // whole-loop kernel of small 2D FP32 grids
   int loop_on = 0;             // 1: propagations run it
+  cudaError_t loop_err = cudaSuccess;   // first launch of it that was refused (take_loop_error)
   int medium_k = 0;            // checkpoint interval of the medium gradient (0: automatic)
 };
 
@@ -609,6 +610,19 @@ bool use_loop(const qpat_ctx* c, int batch) {
   return loop_waves(c->loop, batch) <= 1 || (c->loop.own_kernel && !(c->pf.fast_rows && c->pf.fast_cols));
 }
 
+// A refused launch of the whole-loop kernel, once.  (A cluster launch can be
+// refused while a graph is being captured without ending the capture: the graph
+// would lack the propagation.)
+cudaError_t take_loop_error(qpat_ctx* c) {
+  const cudaError_t e = c->loop_err;
+  if (e != cudaSuccess) cudaGetLastError();
+  c->loop_err = cudaSuccess;
+  return e;
+}
+void loop_launched(qpat_ctx* c, cudaError_t e) {
+  if (c->loop_err == cudaSuccess) c->loop_err = e;
+}
+
 // seq_forward and seq_adjoint on the whole-loop kernel: one launch, or one per
 // checkpoint interval when checkpoints are stored.
 long long seq_loop_forward(qpat_ctx* c, int batch, cudaStream_t s, int K, bool store, int resume_m) {
@@ -625,19 +639,19 @@ long long seq_loop_forward(qpat_ctx* c, int batch, cudaStream_t s, int K, bool s
   if (store && K > 0)
     for (int m = 0; m < (nt - 1) / K; ++m) {
       const int g1 = (m + 1) * K * P;
-      launch_loop(c->pf, c->loop, 0, ll, batch, nt, g, g1, load, 1, 0, 0, s);
+      loop_launched(c, launch_loop(c->pf, c->loop, 0, ll, batch, nt, g, g1, load, 1, 0, 0, s));
       launch_ckpt_copy<float>(c->pf, batch, m, 1, s, layout);
       g = g1;
       load = 1;
       ++cnt;
     }
-  launch_loop(c->pf, c->loop, 0, ll, batch, nt, g, end, load, 0, resume_m >= 0 && ll, 1, s);
+  loop_launched(c, launch_loop(c->pf, c->loop, 0, ll, batch, nt, g, end, load, 0, resume_m >= 0 && ll, 1, s));
   return cnt + 1;
 }
 
 long long seq_loop_adjoint(qpat_ctx* c, int batch, cudaStream_t s) {
   const int ll = c->cfg.lossless != 0;
-  launch_loop(c->pf, c->loop, 1, ll, batch, c->nt, 0, c->nt * (ll ? 4 : 6) - 3, 0, 0, 0, 0, s);
+  loop_launched(c, launch_loop(c->pf, c->loop, 1, ll, batch, c->nt, 0, c->nt * (ll ? 4 : 6) - 3, 0, 0, 0, 0, s));
   return 1;
 }
 
@@ -770,6 +784,8 @@ qpat_status run_prop(qpat_ctx* c, int dir, int batch, const T* p0, T* data, cons
   const bool direct = c->cfg.no_graphs || c->prof_phase >= 0;
   if (direct) {
     c->launches += seq_any(c, dir, batch, c->stream);
+    const cudaError_t e = take_loop_error(c);
+    if (e != cudaSuccess) return cuda_fail(c, e, "propagation kernel");
     QCK(cudaGetLastError());
     return QPAT_OK;
   }
@@ -779,8 +795,14 @@ qpat_status run_prop(qpat_ctx* c, int dir, int batch, const T* p0, T* data, cons
     if (!c->cap_stream) QCK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
     QCK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     const long long n = seq_any(c, dir, batch, c->cap_stream);
+    const cudaError_t launch = take_loop_error(c);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
+    if (launch != cudaSuccess) {
+      if (g) cudaGraphDestroy(g);
+      if (e != cudaSuccess) cudaGetLastError();
+      return cuda_fail(c, launch, "propagation kernel");
+    }
     if (e != cudaSuccess) return cuda_fail(c, e, "graph capture");
     cudaGraphExec_t ex = nullptr;
     e = cudaGraphInstantiate(&ex, g, 0);
@@ -800,6 +822,8 @@ qpat_status run_ckpt(qpat_ctx* c, int batch, const T* p0, T* data, T* ckpt, int 
   IoPtrs<T>* io = const_cast<IoPtrs<T>*>(a.io);
   launch_set_io<T>(io, p0, data, nullptr, nullptr, ckpt, c->stream);
   c->launches += seq_forward<T>(c, batch, c->stream, K, resume_m < 0, resume_m);
+  const cudaError_t e = take_loop_error(c);
+  if (e != cudaSuccess) return cuda_fail(c, e, "propagation kernel");
   QCK(cudaGetLastError());
   return QPAT_OK;
 }
@@ -1491,6 +1515,16 @@ long long seq_group(qpat_group* g, int dir, const int* batches, GroupRun run) {
   return kernels;
 }
 
+// take_loop_error over the members.
+cudaError_t group_loop_error(qpat_group* g) {
+  cudaError_t first = cudaSuccess;
+  for (qpat_ctx* c : g->ctxs) {
+    const cudaError_t e = take_loop_error(c);
+    if (first == cudaSuccess) first = e;
+  }
+  return first;
+}
+
 bool shape_valid(const qpat_group_shape& sh) {
   return (sh.multi == 0 || sh.multi == 1) && (sh.row_block == 144 || sh.row_block == 288) &&
          (sh.col_block == 288 || sh.col_block == 576) && (sh.largest_first == 0 || sh.largest_first == 1);
@@ -1567,8 +1601,14 @@ qpat_status qpat_group_propagate(qpat_group* g, int dir, const int* batches, con
     cudaError_t e = cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(c0, e, "group capture");
     const long long kernels = seq_group(g, dir, batches, run);
+    const cudaError_t launch = group_loop_error(g);
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(g->cap, &graph);
+    if (launch != cudaSuccess) {
+      if (graph) cudaGraphDestroy(graph);
+      if (e != cudaSuccess) cudaGetLastError();
+      return cuda_fail(c0, launch, "group propagation kernel");
+    }
     if (e != cudaSuccess) return cuda_fail(c0, e, "group capture end");
     cudaGraphExec_t ex = nullptr;
     e = cudaGraphInstantiate(&ex, graph, 0);
@@ -1675,7 +1715,9 @@ qpat_status qpat_group_tune(qpat_group* g, const int* batches, int steps, void* 
       cudaError_t e = cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
         seq_group(g, dir, batches, multi ? kMulti : kBranches);
+        const cudaError_t launch = group_loop_error(g);
         e = cudaStreamEndCapture(g->cap, &graph);
+        if (launch != cudaSuccess) e = launch;
       }
       if (e == cudaSuccess) e = cudaGraphInstantiate(&ex[dir], graph, 0);
       if (graph) cudaGraphDestroy(graph);
@@ -1751,6 +1793,7 @@ qpat_status qpat_autotune(qpat_ctx* c, int batch, int steps, int* choice) {
     c->pf.fast_rows = c->pd.fast_rows = fr;
     c->pf.fast_cols = c->pd.fast_cols = fc;
     float total = 0.f;
+    bool refused = false;
     for (int rep = 0; rep < 2; ++rep) {   // first repetition warms up
       if (c->prec == QPAT_FP32) set_io_for<float>(c, 0, p0, data, c->stream);
       else set_io_for<double>(c, 0, p0, data, c->stream);
@@ -1764,7 +1807,9 @@ qpat_status qpat_autotune(qpat_ctx* c, int batch, int steps, int* choice) {
       float ms = 0.f;
       cudaEventElapsedTime(&ms, e0, e1);
       if (rep == 1) total = ms;
+      refused = take_loop_error(c) != cudaSuccess || refused;
     }
+    if (refused) continue;
     if (total < best) { best = total; best_choice = loop ? 3 : cand; best_loop = loop; }
   }
   c->nt = nt_saved;
