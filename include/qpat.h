@@ -280,7 +280,7 @@ qpat_status qpat_group_jvp(qpat_group* group, const int* batches, const double* 
  * col_block: threads per column-pass CTA, 288 or 576 (adjacent columns per
  *   CTA: col_block / 48 or col_block / 72).
  * largest_first: 1 hands the work items of the largest extent to the first
- *   CTAs.  Default {1, 144, 576, 1}.
+ *   CTAs.
  * The shape applies once it has been set or tuned.  Until then the members run
  * their own launch sequences, one after the other where each fills the GPU,
  * else as the branches of multi = 0 (the results are the same bit for bit). */
@@ -294,17 +294,19 @@ typedef struct {
 /* Set the shape of later group calls (EINVAL for values outside the lists). */
 qpat_status qpat_group_set_shape(qpat_group* group, const qpat_group_shape* shape);
 
-/* The present shape; *multi_ready (optional) = 1 when the members with work
+/* The shape that was set or tuned ({1, 144, 576, 1}, which no call follows,
+ * before either); *multi_ready (optional) = 1 when the members with work
  * in `batches` (per member, may be NULL) qualify for multi-problem launches. */
 qpat_status qpat_group_get_shape(const qpat_group* group, qpat_group_shape* shape, int* multi_ready,
                                  const int* batches);
 
 /* Autotuner of the group's launch shape: times a `steps`-step forward +
  * adjoint of batches[i] problems per member (a CUDA graph per direction,
- * second of two runs, CUDA events on `stream`) for multi = 0 and for every
- * multi-problem shape (row_block x col_block x largest_first) when the
- * members qualify, keeps the fastest as the group's shape and returns it in
- * *best.  ms (optional, up to 16 entries) receives each candidate's time in
+ * second of two runs, CUDA events on `stream`) for multi = 0, as branches and
+ * with the members one after the other, and for every multi-problem shape
+ * (row_block x col_block x largest_first) when the members qualify, keeps the
+ * fastest as the group's shape and returns it in *best (of the two forms of
+ * multi = 0 the group keeps the faster, until a shape is set).  ms (optional, up to 16 entries) receives each candidate's time in
  * candidate order (multi = 0 first, then row_block 144/288 x col_block
  * 288/576 x largest_first 1/0); *ncand (optional) their count.  The members'
  * loops are shortened to `steps` during the call.  Allocates and frees

@@ -1301,6 +1301,7 @@ struct qpat_group {
   std::map<std::vector<int>, std::pair<cudaGraphExec_t, long long>> graphs;
   qpat_group_shape shape{1, 144, 576, 1};
   bool chosen = false;         // the shape was set or tuned: group calls follow it
+  bool in_turn = false;        // tuned, multi = 0: the members run one after the other
 };
 
 namespace {
@@ -1479,13 +1480,15 @@ long long seq_multi_adjoint(const std::vector<MMember>& mm, const qpat_group_sha
 // own sequence as a parallel branch, or those sequences one after the other.
 enum GroupRun { kBranches = 0, kMulti = 1, kInTurn = 2 };
 
-// A set or tuned shape is followed.  Without one, members that each fill the
+// A set or tuned shape is followed (tuning also tells whether multi = 0 means
+// branches or in turn).  Without one, members that each fill the
 // chip (a million grid points of all their problems: two rounds of the passes'
 // CTAs) run in turn, others as branches: 16 problems on each of 288^2, 432^2,
 // 576^2, 80 steps, take 30.0 ms in turn, 32.3 as branches (their working sets
 // compete for L2) and 42.4 as multi-problem launches.
 GroupRun group_run(const qpat_group* g, const int* batches) {
-  if (g->chosen) return g->shape.multi && !multi_members(g, batches).empty() ? kMulti : kBranches;
+  if (g->chosen && g->shape.multi) return multi_members(g, batches).empty() ? kBranches : kMulti;
+  if (g->chosen) return g->in_turn ? kInTurn : kBranches;
   for (size_t i = 0; i < g->ctxs.size(); ++i)
     if (batches[i] > 0 && (double)g->ctxs[i]->G * batches[i] < 1e6) return kBranches;
   return kInTurn;
@@ -1644,6 +1647,7 @@ qpat_status qpat_group_set_shape(qpat_group* g, const qpat_group_shape* shape) {
   if (!g || !shape || !shape_valid(*shape)) return QPAT_EINVAL;
   g->shape = *shape;
   g->chosen = true;
+  g->in_turn = false;
   return QPAT_OK;
 }
 
@@ -1666,7 +1670,8 @@ qpat_status qpat_group_tune(qpat_group* g, const int* batches, int steps, void* 
     if (batches[i] < 0 || batches[i] > c->maxb) return fail(c, QPAT_EINVAL, "group batch out of range");
     if (c->prof_phase >= 0) return fail(c, QPAT_EINVAL, "profiling is not available in group calls");
   }
-  std::vector<qpat_group_shape> cand{{0, 144, 576, 1}};
+  // candidate 0, the members' own sequences, is tried as branches and in turn
+  std::vector<qpat_group_shape> cand{{0, 144, 576, 1}, {0, 144, 576, 1}};
   if (!multi_members(g, batches).empty())
     for (int rb : {144, 288})
       for (int cb : {288, 576})
@@ -1708,13 +1713,13 @@ qpat_status qpat_group_tune(qpat_group* g, const int* batches, int steps, void* 
   for (int i = 0; i < n; ++i) g->ctxs[i]->nt = std::max(2, std::min(steps, saved[i]));
   for (size_t k = 0; k < cand.size() && st == QPAT_OK; ++k) {
     g->shape = cand[k];
-    const bool multi = cand[k].multi != 0;
+    const GroupRun run = cand[k].multi ? kMulti : k == 0 ? kBranches : kInTurn;
     cudaGraphExec_t ex[2] = {nullptr, nullptr};
     for (int dir = 0; dir < 2 && st == QPAT_OK; ++dir) {
       cudaGraph_t graph = nullptr;
       cudaError_t e = cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        seq_group(g, dir, batches, multi ? kMulti : kBranches);
+        seq_group(g, dir, batches, run);
         const cudaError_t launch = group_loop_error(g);
         e = cudaStreamEndCapture(g->cap, &graph);
         if (launch != cudaSuccess) e = launch;
@@ -1743,7 +1748,9 @@ qpat_status qpat_group_tune(qpat_group* g, const int* batches, int steps, void* 
     }
     for (cudaGraphExec_t x : ex)
       if (x) cudaGraphExecDestroy(x);
-    if (ms && k < 16) ms[k] = t;
+    if (ms && k == 0) ms[0] = t;
+    else if (ms && k == 1) ms[0] = std::min(ms[0], (double)t);
+    else if (ms && k <= 16) ms[k - 1] = t;
     if (st == QPAT_OK && t < best_ms) {
       best_ms = t;
       best_k = (int)k;
@@ -1753,9 +1760,12 @@ qpat_status qpat_group_tune(qpat_group* g, const int* batches, int steps, void* 
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   g->shape = st == QPAT_OK ? cand[best_k] : keep;
-  g->chosen = g->chosen || st == QPAT_OK;
+  if (st == QPAT_OK) {
+    g->chosen = true;
+    g->in_turn = best_k == 1;
+  }
   if (best) *best = g->shape;
-  if (ncand) *ncand = (int)cand.size();
+  if (ncand) *ncand = (int)cand.size() - 1;
   return st;
 }
 
