@@ -317,8 +317,10 @@ qpat_status qpat_group_tune(qpat_group* group, const int* batches, int steps, vo
 /* Autotuner: time a `steps`-step forward + adjoint of `batch` problems with
  * every supported choice of pass kernels (specialised or generic row passes,
  * specialised or generic column passes) and keep the fastest for this
- * context; *choice = bit 0 rows specialised, bit 1 columns specialised (3
- * also for the whole-loop kernel of small 2D FP32 grids).
+ * context; *choice = bit 0 rows specialised, bit 1 columns specialised.  Where
+ * the grid has a whole-loop kernel (small 2D FP32 grids) it is timed too, and
+ * later calls with this batch run it if it was faster still; other batches keep
+ * their own choice between it and the pass kernels.
  * Synchronises; allocates and frees temporary buffers. */
 qpat_status qpat_autotune(qpat_ctx* ctx, int batch, int steps, int* choice);
 

@@ -63,7 +63,8 @@ struct qpat_ctx {
   std::vector<cudaEvent_t> prof_events;
   size_t prof_used = 0;
   LoopPlan loop;               // whole-loop kernel of small 2D FP32 grids
-  int loop_on = 0;             // 1: propagations run it
+  bool loop_beyond = false;    // runs it also for more problems than fit at once (use_loop)
+  std::map<int, bool> loop_tuned;   // per batch that qpat_autotune was given: whether it was the faster
   cudaError_t loop_err = cudaSuccess;   // first launch of it that was refused (take_loop_error)
   int medium_k = 0;            // checkpoint interval of the medium gradient (0: automatic)
 };
@@ -560,7 +561,7 @@ qpat_status build_context(qpat_ctx* c, const qpat_medium* med, const double* sen
   if constexpr (std::is_same<T, float>::value) {
     // (cfg.generic_fft asks for the generic passes)
     if (!c->cfg.generic_fft) loop_plan(a, c->cfg.lossless, c->maxb, &c->loop);
-    c->loop_on = c->loop.ok;
+    c->loop_beyond = c->loop.own_kernel && !(a.fast_rows && a.fast_cols);
   }
   return QPAT_OK;
 }
@@ -603,11 +604,13 @@ void pass(qpat_ctx* c, const PropArgs<T>& a, int phase, int batch, bool is_row, 
 // length-specialised form.  (100 steps, forward + adjoint, loop kernel against
 // launched passes, ms: 168^2, specialised passes, 6 problems 4.3 / 6.8, 8
 // 8.6 / 6.9; 200^2 4 5.0 / 9.6, 32 25.1 / 33.3; 216 x 168 4 6.8 / 7.2, 16
-// 20.2 / 13.3.)  The pass profiler times single passes, so it sees the
-// launched ones.
+// 20.2 / 13.3.)  What qpat_autotune measured at a batch decides for that batch.
+// The pass profiler times single passes, so it sees the launched ones.
 bool use_loop(const qpat_ctx* c, int batch) {
-  if (!c->loop_on || c->prof_phase >= 0) return false;
-  return loop_waves(c->loop, batch) <= 1 || (c->loop.own_kernel && !(c->pf.fast_rows && c->pf.fast_cols));
+  if (!c->loop.ok || c->prof_phase >= 0) return false;
+  const auto it = c->loop_tuned.find(batch);
+  if (it != c->loop_tuned.end()) return it->second;
+  return loop_waves(c->loop, batch) <= 1 || c->loop_beyond;
 }
 
 // A refused launch of the whole-loop kernel, once.  (A cluster launch can be
@@ -1797,11 +1800,12 @@ qpat_status qpat_autotune(qpat_ctx* c, int batch, int steps, int* choice) {
   for (int cand = 0; cand < 5; ++cand) {
     const bool loop = cand == 4;                // the whole-loop kernel, last
     const int fr = cand & 1, fc = (cand >> 1) & 1;
-    if (!loop && ((fr && !rows_ok) || (fc && !cols_ok))) continue;
-    c->loop_on = loop && c->loop.ok;
-    if (loop && !use_loop(c, batch)) continue;
-    c->pf.fast_rows = c->pd.fast_rows = fr;
-    c->pf.fast_cols = c->pd.fast_cols = fc;
+    if (loop ? !c->loop.ok : (fr && !rows_ok) || (fc && !cols_ok)) continue;
+    if (c->loop.ok) c->loop_tuned[batch] = loop;
+    if (!loop) {
+      c->pf.fast_rows = c->pd.fast_rows = fr;
+      c->pf.fast_cols = c->pd.fast_cols = fc;
+    }
     float total = 0.f;
     bool refused = false;
     for (int rep = 0; rep < 2; ++rep) {   // first repetition warms up
@@ -1820,11 +1824,14 @@ qpat_status qpat_autotune(qpat_ctx* c, int batch, int steps, int* choice) {
       refused = take_loop_error(c) != cudaSuccess || refused;
     }
     if (refused) continue;
-    if (total < best) { best = total; best_choice = loop ? 3 : cand; best_loop = loop; }
+    if (total < best) {
+      best = total;
+      best_loop = loop;
+      if (!loop) best_choice = cand;
+    }
   }
   c->nt = nt_saved;
-  c->loop_on = best_loop;
-  if (best_loop) best_choice = 3;
+  if (c->loop.ok) c->loop_tuned[batch] = best_loop;
   c->pf.fast_rows = c->pd.fast_rows = rows_ok && (best_choice & 1);
   c->pf.fast_cols = c->pd.fast_cols = cols_ok && ((best_choice >> 1) & 1);
   for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second.first);
