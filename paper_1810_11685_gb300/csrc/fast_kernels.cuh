@@ -20,11 +20,19 @@
 namespace qpat {
 
 // Forward radix plans (Q3 = 1: two stages).  The inverse uses them reversed.
+// Two stages of a short extent leave few threads a transform, each with a long
+// serial chain; three cost one more barrier.  All five short extents were measured
+// both ways, in several orders of the radices; three stages are taken where they
+// are faster and their error against 64 bits is no larger (100 steps, forward +
+// adjoint, ms, two stages -> three, and the error's factor): 24 = 4 3 2: 24^3
+// 7.63 -> 6.66, 24^2 x 512 7.04 -> 6.35, 0.94 (2 3 4: 6.38 and 5.28, but up to
+// 1.03); 48 = 4 3 4: 48^3 9.08 -> 7.56, 48^2 x 128 5.50 -> 5.11, x 256 7.15 ->
+// 7.46, 0.87 (3 4 4: 7.39, 4.82 and 6.31, 0.97).  Not: 40 = 2 5 4, 40^2 x 256
+// 6.08 -> 6.86; 54 = 3 6 3, 54^2 x 256 10.7 -> 8.6, but 1.02; 56 = 2 7 4, 56^2 x
+// 256 10.8 -> 11.1.
 template <int L> struct SPlan { static constexpr int Q1 = 0, Q2 = 0, Q3 = 0; };
-template <> struct SPlan<24> { static constexpr int Q1 = 4, Q2 = 6, Q3 = 1; };
+template <> struct SPlan<24> { static constexpr int Q1 = 4, Q2 = 3, Q3 = 2; };
 template <> struct SPlan<40> { static constexpr int Q1 = 5, Q2 = 8, Q3 = 1; };
-// (three stages for 48: two of radix 6 and 8 left 8 threads a transform with a long serial chain; 48^3 x 3, 150
-// steps, forward + adjoint 16.8 -> 14.9 ms)
 template <> struct SPlan<48> { static constexpr int Q1 = 4, Q2 = 3, Q3 = 4; };
 template <> struct SPlan<54> { static constexpr int Q1 = 6, Q2 = 9, Q3 = 1; };
 template <> struct SPlan<56> { static constexpr int Q1 = 7, Q2 = 8, Q3 = 1; };
