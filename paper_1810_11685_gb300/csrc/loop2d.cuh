@@ -891,6 +891,21 @@ cudaError_t loop_launch_one(const LoopArgs& A, int nc, int batch, size_t smem, c
       return ll ? loop_occupancy_one<true, true, L>(nc, smem) : loop_occupancy_one<true, false, L>(nc, smem); \
     return ll ? loop_occupancy_one<false, true, L>(nc, smem) : loop_occupancy_one<false, false, L>(nc, smem); \
   }
+// Extent L without absorption only: with it the loop's data of a rank of sixteen
+// is above the 227 KB of shared memory a CTA may use (loop_layout; 244 KB at 224).
+#define QPAT_LOOP_INST_LOSSLESS(L)                                                                     \
+  template <>                                                                                          \
+  cudaError_t loop_launch_len<L>(const LoopArgs& A, int adj, int ll, int nc, int batch, size_t smem,   \
+                                 cudaStream_t s) {                                                     \
+    if (!ll) return cudaErrorInvalidValue;                                                             \
+    return adj ? loop_launch_one<true, true, L>(A, nc, batch, smem, s)                                 \
+               : loop_launch_one<false, true, L>(A, nc, batch, smem, s);                               \
+  }                                                                                                    \
+  template <>                                                                                          \
+  int loop_occupancy_len<L>(int adj, int ll, int nc, size_t smem) {                                    \
+    if (!ll) return 0;                                                                                 \
+    return adj ? loop_occupancy_one<true, true, L>(nc, smem) : loop_occupancy_one<false, true, L>(nc, smem); \
+  }
 #define QPAT_LOOP_INST0(ADJ, LL)                                                                       \
   template int loop_occupancy_one<ADJ, LL, 0>(int, size_t);                                            \
   template cudaError_t loop_launch_one<ADJ, LL, 0>(const LoopArgs&, int, int, size_t, cudaStream_t);

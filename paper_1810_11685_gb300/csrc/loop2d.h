@@ -88,7 +88,7 @@ __host__ __device__ inline LoopLayout loop_layout(const LoopAxis& x, const LoopA
   l.total = l.pml + loop_r4(2 * (size_t)x.L + 4 * (size_t)rp);
   return l;
 }
-// Extents with kernels of their own (square grids); the others, and uneven
+// Extents with kernels of their own (square grids; 224 without absorption only); the others, and uneven
 // grids, run the kernels for runtime lengths.
 #define QPAT_LOOP_EXTENTS(X) \
   X(24) X(30) X(32) X(36) X(40) X(42) X(48) X(50) X(54) X(56) X(60) X(64) \
