@@ -133,7 +133,12 @@ qpat_status qpat_sync(qpat_ctx* ctx);
 
 /* H_a (Section 3.2.3): batch of initial pressures -> sensor series.
  * p0:   device prec [batch][N] interior initial pressure (0 in the PML).
- * data: device prec [batch][nt][ns] output.  1 <= batch <= max_batch. */
+ * data: device prec [batch][nt][ns] output.  1 <= batch <= max_batch.
+ * A problem's result does not depend on the other problems of its batch.  Its
+ * last bits may depend on their number, on small 2D FP32 grids: a batch whose
+ * problems fit the GPU at once runs a kernel for the whole loop, a larger one
+ * the passes one by one (or as qpat_autotune found faster), and the two round
+ * differently.  Contexts with generic_fft = 1 always run the same passes. */
 qpat_status qpat_acoustic_forward(qpat_ctx* ctx, int batch, const void* p0, void* data);
 
 /* H_a^* (Lemma 2, eq. t41, computed as the exact transpose of H_a).

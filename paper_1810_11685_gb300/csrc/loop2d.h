@@ -89,7 +89,10 @@ __host__ __device__ inline LoopLayout loop_layout(const LoopAxis& x, const LoopA
   return l;
 }
 // Extents with kernels of their own (square grids; 224 without absorption only); the others, and uneven
-// grids, run the kernels for runtime lengths.
+// grids, run the kernels for runtime lengths.  (Both on the same square grid, one
+// problem, 200 steps, forward + adjoint, runtime / compile-time length, ms: 56^2
+// 9.19 / 5.71, 96^2 8.96 / 5.81, 120^2 10.1 / 6.34, 168^2 12.2 / 8.78, 210^2
+// 14.7 / 11.3.)
 #define QPAT_LOOP_EXTENTS(X) \
   X(24) X(30) X(32) X(36) X(40) X(42) X(48) X(50) X(54) X(56) X(60) X(64) \
   X(70) X(72) X(80) X(84) X(90) X(96) X(98) X(100) X(108) X(112) X(120) X(126) \
