@@ -14,6 +14,7 @@ int line_stride(const LoopAxis& x, const LoopAxis& y) {
 }
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
 constexpr int kClusters[3] = {16, 8, 4};
+constexpr size_t kMaxSmem = 227 * 1024;
 }  // namespace
 
 size_t loop_smem(const PropArgs<float>& a, const LoopAxis& x, const LoopAxis& y, int nc, int adj, int lossless) {
@@ -66,36 +67,65 @@ void loop_plan(const PropArgs<float>& a, int lossless, int max_batch, LoopPlan* 
   if (!p->x.L || !p->y.L) return;
   const int L = kernel_extent(a);
   p->own_kernel = L != 0;
-  // the adjoint kernel holds more than the forward one: it decides the fit
-  // (smaller clusters are only looked at when max_batch may not fit as 16s)
-  if (!occupancy(L, 0, lossless, 0, 0)) return;
+  p->specialised = a.fast_rows && a.fast_cols;
+  bool two_power = true;
+  for (const LoopAxis* x : {&p->x, &p->y})
+    for (int q : x->q) two_power = two_power && (q == 2 || q == 4 || q == 8);
+  p->shared_cost = !p->specialised && (lossless || two_power) ? 1.1 : 1.5;
+  // (also sets both kernels' attributes; the adjoint kernel holds more than the
+  // forward one and decides the fit)
+  if (!occupancy(L, 0, lossless, 0, 0) || !occupancy(L, 1, lossless, 0, 0)) return;
   for (int k = 0; k < 3; ++k) {
-    p->max_clusters[k] = occupancy(L, 1, lossless, kClusters[k], loop_smem(a, p->x, p->y, kClusters[k], 1, lossless));
-    p->ok = p->ok || p->max_clusters[k] > 0;
-    if (k == 0 && p->max_clusters[0] >= max_batch) break;
+    const size_t smem = loop_smem(a, p->x, p->y, kClusters[k], 1, lossless);
+    if (smem > kMaxSmem) break;                                  // (smaller clusters need more)
+    p->alone[k] = occupancy(L, 1, lossless, kClusters[k], kMaxSmem);
+    p->ok = p->ok || p->alone[k] > 0;
+    if (p->alone[k] >= max_batch && k == 0) {                    // no more looked up than max_batch may need
+      p->max_clusters[k] = p->alone[k];
+      break;
+    }
+    p->max_clusters[k] = occupancy(L, 1, lossless, kClusters[k], smem);
   }
 }
 
 namespace {
-// Cluster size (index into kClusters) for `batch` problems: the fewest rounds
-// of resident clusters, weighted by the time of a step (96^2: 16 CTAs 14.6 us,
-// 8 16.7 us, 4 23.4 us); 16 for one round.
+double points_per_cta(const LoopPlan& p, int k) { return (double)p.x.L * p.y.L / kClusters[k]; }
+// Cluster size (index into kClusters) for `batch` problems, by the time of a
+// step: the passes' latency and the points of a CTA, times the rounds of resident
+// clusters.  A round in which two CTAs share an SM measured 1.5 rounds with
+// absorption, 1.0 to 1.16 without or with radices 2, 4 and 8 only (54^2 and 56^2
+// without: 1.5, so grids with specialised passes, whose smaller clusters cost
+// nothing, always count 1.5).  24 steps, forward + adjoint, clusters of 16 / 8 / 4,
+// ms; alone on the SMs are 7, 15 and 36 clusters: 40^2, one problem 0.67 / 0.67 /
+// 0.67, 12 1.00 / 0.69 / 0.69, 32 2.60 / 1.33 / 0.70; 64^2 x 12 0.74 / 0.70 / 0.75;
+// 96^2, one problem 0.73 / 0.84 / 1.16, 16 1.81 / 1.27 / 1.17; 120^2 x 32 lossless
+// 1.73 / 1.34 / 1.00.  (Counting rounds of resident clusters alone took 40^2 x 32
+// in clusters of 8, behind the launched passes' 1.14.)
 int choose(const LoopPlan& p, int batch) {
-  static const double cost[3] = {1.0, 1.15, 1.6};
+  const double flat = p.own_kernel ? 2600.0 : 6000.0;           // points of a CTA that take as long as the rest of a step
   int k = -1;
   double best = 1e300;
   for (int q = 0; q < 3; ++q) {
-    if (p.max_clusters[q] <= 0) continue;
-    const double c = cost[q] * ceil_div(batch, p.max_clusters[q]);
+    const int n = p.max_clusters[q];
+    if (n <= 0) continue;
+    const int rest = batch % n;
+    const double full = n > p.alone[q] ? p.shared_cost : 1.0;
+    const double rounds = batch / n * full + (rest == 0 ? 0.0 : rest > p.alone[q] ? full : 1.0);
+    const double c = (1.0 + points_per_cta(p, q) / flat) * rounds;
     if (c < best) { best = c; k = q; }
   }
   return k;
 }
 }  // namespace
 
+// (Where the launched passes are specialised on both axes they are the faster
+// against smaller clusters of many points a CTA: 168^2 x 12 lossless, 24 steps,
+// clusters of 8 with 3528 points 1.08 ms, launched 1.05; 168 x 48 x 24 lossless,
+// clusters of 4 with 2016 0.99 / 0.89; 56^2 x 32, clusters of 4 with 784 0.76 / 1.30.)
 int loop_waves(const LoopPlan& p, int batch) {
   const int k = choose(p, batch);
-  return k < 0 ? 1 << 30 : ceil_div(batch, p.max_clusters[k]);
+  if (k < 0 || (p.specialised && k > 0 && points_per_cta(p, k) > 1024.0)) return 1 << 30;
+  return ceil_div(batch, p.max_clusters[k]);
 }
 
 cudaError_t launch_loop(const PropArgs<float>& a, const LoopPlan& p, int adj, int lossless, int batch, int nt, int g0,

@@ -54,7 +54,10 @@ struct LoopPlan {
   int ok = 0;              // the grid has a plan and one problem fits a cluster
   int own_kernel = 0;      // square grid of an extent with compile-time kernels
   LoopAxis x{}, y{};
-  int max_clusters[3] = {0, 0, 0}; // clusters of 16, 8, 4 CTAs resident at once (0: does not fit)
+  bool specialised = false;  // the launched passes are specialised on both axes
+  double shared_cost = 1.0;  // time of a round with two CTAs to an SM against one with one
+  int alone[3] = {0, 0, 0};  // clusters of 16, 8, 4 CTAs resident with one CTA to an SM (0: does not fit)
+  int max_clusters[3] = {0, 0, 0}; // clusters resident at once
 };
 
 struct LoopArgs {
@@ -104,7 +107,8 @@ __host__ __device__ inline LoopLayout loop_layout(const LoopAxis& x, const LoopA
 size_t loop_smem(const PropArgs<float>& a, const LoopAxis& x, const LoopAxis& y, int nc, int adj, int lossless);
 // Plan of a grid; sets the kernels' attributes.
 void loop_plan(const PropArgs<float>& a, int lossless, int max_batch, LoopPlan* p);
-// Rounds of resident clusters that `batch` problems take.
+// Rounds of resident clusters that `batch` problems take; more than any
+// number where the launched passes are known to be faster.
 int loop_waves(const LoopPlan& p, int batch);
 // Passes [g0, g1) of H_a (adj = 0) or H_a^* (adj = 1) of nt samples for
 // `batch` problems.
