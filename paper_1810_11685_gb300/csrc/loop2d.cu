@@ -102,7 +102,8 @@ double points_per_cta(const LoopPlan& p, int k) { return (double)p.x.L * p.y.L /
 // 1.73 / 1.34 / 1.00.  (Counting rounds of resident clusters alone took 40^2 x 32
 // in clusters of 8, behind the launched passes' 1.14.)
 int choose(const LoopPlan& p, int batch) {
-  const double flat = p.own_kernel ? 2600.0 : 6000.0;           // points of a CTA that take as long as the rest of a step
+  // points of a CTA that take as long as the rest of a step
+  const double flat = p.own_kernel ? 2600.0 : 6000.0;
   int k = -1;
   double best = 1e300;
   for (int q = 0; q < 3; ++q) {
