@@ -65,14 +65,75 @@ constexpr int first_factor(int N) {
        : (N % 7 == 0 && N != 7) ? 7 : N;
 }
 
+// ---- constants of two floats ---------------------------------------------------
+// sqrt(3)/2 and sin(2 pi / 5) as single floats are off by 1.8e-8 and 2.5e-8.  That
+// is the same in every transform, so a time loop's fields shrink or grow by it step
+// after step: over 150 steps it, and the rounding of the twiddles, are most of
+// the error against 64 bits, which then depends on which radices a length is
+// split into: the whole-loop kernel had 1.25 times the error of passes with other
+// radices at 60^2, 1.24 at 108^2, 0.66 at 112^2.  With these constants as two floats
+// it has 0.78 times theirs in the mean over 36 square extents and at most 1.04, for
+// 0.5% of its time.  (cos(2 pi / 5) and cos(4 pi / 5) as -1/4 +- sqrt(5)/4:
+// one constant, exact in their sum.)  Not in the launched passes: there the same
+// constants cost 1% and the rounding of the twiddles, which they leave, is no longer
+// offset at many lengths (400^2 0.82 of the error, 360^2 1.22, 900^2 1.35).
+// A constant as the sum of two floats, and fma(x, c, t) with it.
+struct Const2 {
+  float hi, lo;
+};
+constexpr Const2 const2(double v) { return Const2{(float)v, (float)(v - (double)(float)v)}; }
+template <typename R>
+__device__ __forceinline__ R fma2(R x, Const2 c, R t) {
+  const R u = t + x * (R)c.lo;
+  return u + x * (R)c.hi;
+}
+template <typename R>
+__device__ __forceinline__ R mul2(R x, Const2 c) {
+  const R u = x * (R)c.lo;
+  return u + x * (R)c.hi;
+}
+// dft3 and dft5 with constants of two floats.
+template <typename C>
+__device__ __forceinline__ void dft3_fine(C* a) {
+  typedef decltype(C().x) R;
+  constexpr Const2 h = const2(0.8660254037844386467637231707529362);   // sqrt(3)/2
+  const C t1 = cadd(a[1], a[2]), t2 = csub(a[1], a[2]);
+  const C m = cmake<C>(a[0].x - (R)0.5f * t1.x, a[0].y - (R)0.5f * t1.y);
+  const C s = cmul_mi(cmake<C>(mul2<R>(t2.x, h), mul2<R>(t2.y, h)));
+  a[0] = cadd(a[0], t1);
+  a[1] = cadd(m, s);
+  a[2] = csub(m, s);
+}
+template <typename C>
+__device__ __forceinline__ void dft5_fine(C* a) {
+  typedef decltype(C().x) R;
+  const R k = (R)0.5590169943749474241022934171828191f;                // sqrt(5)/4, (cos(2 pi / 5) - cos(4 pi / 5))/2
+  constexpr Const2 s1 = const2(0.9510565162951535721164393333793821), s2 = const2(0.5877852522924731291687059546390728),
+                   ns1 = const2(-0.9510565162951535721164393333793821);
+  const C b1 = cadd(a[1], a[4]), b2 = cadd(a[2], a[3]), p = cadd(b1, b2), q = csub(b1, b2);
+  const C d1 = csub(a[1], a[4]), d2 = csub(a[2], a[3]);
+  const C m = cmake<C>(a[0].x - (R)0.25f * p.x, a[0].y - (R)0.25f * p.y);
+  const C m1 = cmake<C>(m.x + k * q.x, m.y + k * q.y), m2 = cmake<C>(m.x - k * q.x, m.y - k * q.y);
+  const C n1 = cmul_mi(cmake<C>(fma2<R>(d2.x, s2, mul2<R>(d1.x, s1)), fma2<R>(d2.y, s2, mul2<R>(d1.y, s1))));
+  const C n2 = cmul_mi(cmake<C>(fma2<R>(d2.x, ns1, mul2<R>(d1.x, s2)), fma2<R>(d2.y, ns1, mul2<R>(d1.y, s2))));
+  a[0] = cadd(a[0], p);
+  a[1] = cadd(m1, n1);
+  a[4] = csub(m1, n1);
+  a[2] = cadd(m2, n2);
+  a[3] = csub(m2, n2);
+}
+
 // In-place forward DFT of a[0..N-1] held in registers, natural order in and out.
-template <int N, typename C>
+// FINE: constants of two floats in the factors 3 and 5 and the twiddles of 6.
+template <int N, bool FINE = false, typename C>
 __device__ __forceinline__ void dft(C (&a)[N]) {
   typedef decltype(C().x) R;
   if constexpr (N == 1) {
   } else if constexpr (N == 2) { dft2(a);
+  } else if constexpr (N == 3 && FINE) { dft3_fine(a);
   } else if constexpr (N == 3) { dft3(a);
   } else if constexpr (N == 4) { dft4(a);
+  } else if constexpr (N == 5 && FINE) { dft5_fine(a);
   } else if constexpr (N == 5) { dft5(a);
   } else if constexpr (N == 7) { dft7(a);
   } else if constexpr (N == 8) { dft8(a);
@@ -87,7 +148,7 @@ __device__ __forceinline__ void dft(C (&a)[N]) {
       C t[P];
 #pragma unroll
       for (int n1 = 0; n1 < P; ++n1) t[n1] = a[M * n1 + n2];
-      dft<P>(t);
+      dft<P, FINE>(t);
 #pragma unroll
       for (int k1 = 0; k1 < P; ++k1) y[n2][k1] = t[k1];
     }
@@ -98,7 +159,13 @@ __device__ __forceinline__ void dft(C (&a)[N]) {
         constexpr int k1 = decltype(k1c)::value;
         constexpr double c = cos2pi(n2 * k1, N);
         constexpr double s = sin2pi(n2 * k1, N);
-        y[n2][k1] = cmul(y[n2][k1], cmake<C>((R)c, (R)(-s)));
+        if constexpr (FINE && N == 6) {                  // (cos is 1/2, exact)
+          constexpr Const2 sp = const2(s), sm = const2(-s);
+          const C v = y[n2][k1];
+          y[n2][k1] = cmake<C>(fma2<R>(v.y, sp, v.x * (R)(float)c), fma2<R>(v.x, sm, v.y * (R)(float)c));
+        } else {
+          y[n2][k1] = cmul(y[n2][k1], cmake<C>((R)c, (R)(-s)));
+        }
       });
     });
     // M-point DFTs over n2; output index k1 + P k2
@@ -107,7 +174,7 @@ __device__ __forceinline__ void dft(C (&a)[N]) {
       C u[M];
 #pragma unroll
       for (int n2 = 0; n2 < M; ++n2) u[n2] = y[n2][k1];
-      dft<M>(u);
+      dft<M, FINE>(u);
 #pragma unroll
       for (int k2 = 0; k2 < M; ++k2) a[k1 + P * k2] = u[k2];
     }
