@@ -32,7 +32,8 @@ def errors(shape, pml, lossless):
         ctx = Context(c, rho, None if lossless else np.full(full, 0.75), np.full(shape, 5e-4), sensors, dx=DX,
                       dt=0.3 * DX / c.max(), nt=NT, pml=pml, y=1.5, lossless=lossless, precision=prec,
                       generic_fft=generic)
-        out[name] = [to_np(ctx.acoustic_forward(to_gpu(p0, ctx.dtype))), to_np(ctx.acoustic_adjoint(to_gpu(W, ctx.dtype)))]
+        out[name] = [to_np(ctx.acoustic_forward(to_gpu(p0, ctx.dtype))),
+                     to_np(ctx.acoustic_adjoint(to_gpu(W, ctx.dtype)))]
         ctx.sync()
         ctx.close()
     return [[rel_l2(a, e) for a, e in zip(out[k], out["exact"])] for k in ("loop", "passes")]
