@@ -73,7 +73,8 @@ constexpr int first_factor(int N) {
 // split into: the whole-loop kernel had 1.25 times the error of passes with other
 // radices at 60^2, 1.24 at 108^2, 0.66 at 112^2.  With these constants as two floats
 // it has 0.78 times theirs in the mean over 36 square extents and at most 1.04, for
-// 0.5% of its time.  (cos(2 pi / 5) and cos(4 pi / 5) as -1/4 +- sqrt(5)/4:
+// 0.5% of its time (at runtime lengths, which had 0.92 to 1.04 without, they cost 2
+// to 4% and are left out).  (cos(2 pi / 5) and cos(4 pi / 5) as -1/4 +- sqrt(5)/4:
 // one constant, exact in their sum.)  Not in the launched passes: there the same
 // constants cost 1% and the rounding of the twiddles, which they leave, is no longer
 // offset at many lengths (400^2 0.82 of the error, 360^2 1.22, 900^2 1.35).

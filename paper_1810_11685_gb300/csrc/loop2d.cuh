@@ -262,7 +262,7 @@ __device__ __forceinline__ void first_stage(const LoopCtx& c) {
     E v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = load_point<KIND>(c, m, j + r * nb, L);
-    dft<R, true>(v);
+    dft<R, LC != 0>(v);
     float4* line = c.dst + m * c.stride;
 #pragma unroll
     for (int r = 0; r < R; ++r) put(line, j + r * pitch, v[r]);
@@ -282,7 +282,7 @@ __device__ __forceinline__ void mid_stage(const LoopCtx& c, int RF, const float2
     gather_operands<LC, R, true>(c, c.src + m * c.stride, j, RF, pitch, v);
 #pragma unroll
     for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[(r - 1) * RF + k]);
-    dft<R, true>(v);
+    dft<R, LC != 0>(v);
     float4* out = c.dst + m * c.stride;
     const int o = q * RF * R + k;
 #pragma unroll
@@ -304,7 +304,7 @@ __device__ __forceinline__ void last_stage(const LoopCtx& c, const float2* tw) {
     gather_operands<LC, R, false>(c, c.src + m * c.stride, j, 0, 0, v);
 #pragma unroll
     for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[(r - 1) * nb + j]);
-    dft<R, true>(v);
+    dft<R, LC != 0>(v);
 #pragma unroll
     for (int r = 0; r < R; ++r) store_point<KIND>(c, m, j + r * nb, v[r]);
   }
@@ -479,7 +479,7 @@ __device__ __forceinline__ void point_stage(const LoopArgs& A, const LoopShared&
       gather_operands<LC, R, false>(c, c.src + m * c.stride, j, 0, 0, v);
 #pragma unroll
       for (int r = 1; r < R; ++r) v[r] = cmul(v[r], tw[(r - 1) * nb + j]);
-      dft<R, true>(v);
+      dft<R, LC != 0>(v);
     }
     Eo o[R];
     if constexpr (row) {
@@ -513,7 +513,7 @@ __device__ __forceinline__ void point_stage(const LoopArgs& A, const LoopShared&
       }
     }
     if (!(flags & kSkipOutput)) {
-      dft<R, true>(o);
+      dft<R, LC != 0>(o);
       float4* out = c.dst + m * c.stride;
 #pragma unroll
       for (int r = 0; r < R; ++r) put(out, j + r * pitch, o[r]);
