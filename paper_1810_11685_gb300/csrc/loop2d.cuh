@@ -11,8 +11,8 @@
 // bound by its chain of five barriers, the write-out before the cluster
 // barrier (15% of the warps' time) and the load from L2 behind it.  Measured on
 // GB300, forward + adjoint, launched passes against this: 168^2, one problem,
-// 400 steps 25.8 -> 17.5 ms; 96^2, 200 steps 18.6 -> 5.8 ms; 120^2 x 4, Jacobian
-// product over 400 steps 16.6 -> 7.3 ms; 150 x 210 lossless x 2 (runtime
+// 400 steps 25.8 -> 17.6 ms; 96^2, 200 steps 18.6 -> 5.8 ms; 120^2 x 4, Jacobian
+// product over 400 steps 16.6 -> 7.4 ms; 150 x 210 lossless x 2 (runtime
 // lengths), 200 steps 10.8 -> 8.3 ms.
 //
 // Layout.  Two real fields f0, f1 travel as one complex field f0 + i f1, so a
